@@ -81,7 +81,7 @@ static int fft_factor(int n, int *rad)
 } // namespace supcg
 
 // ------------------------------------------------------------------ objects
-enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWD2, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_TV, KT_COUNT };
+enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWD2, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
 
 struct Workspace {
     int count = 0;
@@ -96,6 +96,7 @@ struct Workspace {
     int bw_max = 0;
     int bparts = 0;             // view parts of every problem's backprojector, 0 if they differ
     int mirror = 0;             // 1: some problem has mirror pairs of views
+    int stv_ti = 0;             // rows of k_stv_tile's tiles; 0: the images do not fit, S_TV walks them in memory
     std::vector<void *> allocs;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t body_exec = nullptr;
@@ -605,11 +606,26 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         npx[c] = (long long)g->nx * g->ny;
         nb[KT_STV][c] = (int)std::max(1LL, std::min<long long>((npx[c] + 1023) / 1024, stv_cap));
         stv_want += nb[KT_STV][c];
+        nb[KT_STVT][c] = 0;
         nb[KT_TV][c] = (int)std::max(1LL, std::min<long long>((npx[c] + 1023) / 1024, 4096));
         w->hp[c].fft_rpb = rpb;
         w->hp[c].fft_cw = cw;
     }
     if (w->smem_rows > 200 * 1024 || w->smem_cols > 200 * 1024) { delete w; return SUPCG_ERR_UNSUPPORTED; }
+    // S_TV on resident tiles when all of them fit the device at once, in the lowest tiles that do (32, 64 or 128
+    // rows; two blocks per SM).  Lower tiles have less work per block between two barriers: K = 40 at 384^2
+    // takes 289, 329 and 426 us with them, at 512^2 338, 338 and 426; where only 64 and 128 rows fit, 640^2
+    // 412 and 429; where only 128 do, 1024^2 569.  In memory: 723, 853, 974 and 1308 us.
+    for (int ti : {32, 64, 128}) {
+        long long tiles = 0;
+        int cap = 0;
+        for (int c = 0; c < w->count; ++c) tiles += stv_tiles(gs[c]->nx, gs[c]->ny, ti);
+        if ((rc = stv_tile_max_blocks(ti, &cap))) { delete w; return rc; }
+        if (tiles > cap) continue;
+        w->stv_ti = ti;
+        for (int c = 0; c < w->count; ++c) nb[KT_STVT][c] = stv_tiles(gs[c]->nx, gs[c]->ny, ti);
+        break;
+    }
     // co-residency of the cooperative S_TV launch: scale down to the device capacity
     // (proportional shares, at least one block each; the rounding-up of the minimum is
     // taken back from the largest shares)
@@ -651,7 +667,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         const size_t mir = g->npairs > 0 ? 1 : 0;   // mirrored images only with mirror pairs
         int maxblk = 0;
         for (int kt = 0; kt < KT_COUNT; ++kt) maxblk = std::max(maxblk, nb[kt][c]);
-        const size_t npart = std::max<size_t>(12 * (size_t)nb[KT_STV][c], 2 * (size_t)maxblk) + 64;
+        const size_t npart = std::max<size_t>(std::max(12 * (size_t)nb[KT_STV][c], 4 * (size_t)nb[KT_STVT][c]), 2 * (size_t)maxblk) + 64;
         auto al = [](size_t b) { return (b + 255) / 256 * 256; };
         const size_t sizes[] = {img * 4, imgT * 4, img * 4, imgT * 4, img * 4, img * 4, img * 4, img * 4,
                                 sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, sizeof(Scal),
@@ -775,6 +791,15 @@ static int ws_upload(Workspace *w, cudaStream_t st)
     SUPCG_CUDA_TRY(cudaStreamSynchronize(st));
     SUPCG_CUDA_TRY(cudaMemcpy(w->dp, w->hp.data(), sizeof(Prob) * w->count, cudaMemcpyHostToDevice));
     return SUPCG_OK;
+}
+
+// S_TV over the problems of w: on resident tiles where they fit and no learned direction is given.
+static int enqueue_stv(Workspace *w, cudaStream_t st, int K, double a, double gamma, long long max_trials, int *trials_out,
+                       int want_snorm, const float *dir = nullptr)
+{
+    if (w->stv_ti && !dir && K > 0)
+        return launch_stv_tile(w->L(KT_STVT, st), w->stv_ti, K, a, gamma, max_trials, trials_out, want_snorm);
+    return launch_stv(w->L(KT_STV, st), K, a, gamma, max_trials, trials_out, want_snorm, dir);
 }
 
 static int ops_ws(supcg_geometry g, int batch, Workspace **out)
@@ -931,9 +956,9 @@ extern "C" int supcg_superiorize(supcg_geometry g, float *d_x, double a, double 
     Scal s0 = {};
     s0.ell = *h_ell;
     SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 2 * sizeof(unsigned), st));
+    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
     if ((rc = launch_stage_in(w->L(KT_TR, st), 0))) return rc;
-    if ((rc = launch_stv(w->L(KT_STV, st), K, a, gamma, max_trials, K > 0 ? w->trials_dev : nullptr, 0))) return rc;
+    if ((rc = enqueue_stv(w, st, K, a, gamma, max_trials, K > 0 ? w->trials_dev : nullptr, 0))) return rc;
     if ((rc = launch_store_out(w->L(KT_VEC, st), 0))) return rc;
     Scal s;
     if ((rc = read_scal(P, &s, st))) return rc;
@@ -1021,7 +1046,7 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
     Scal s0 = {};
     s0.muX = isnan(p->mu) ? 0.0 : p->mu;
     SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 2 * sizeof(unsigned), st));
+    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
     SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st), 1));   // b -> bpad
     if (isnan(p->mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
@@ -1036,7 +1061,7 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
             LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, p->cycles, p->r, p->lambda, g->art_S, blocks, st));
     } else {
         for (int c = 0; c < p->cycles; ++c) {   // SupART: S_TV, then one cycle
-            LAUNCH(SUPCG_KIND_STV, st, launch_stv(w->L(KT_STV, st), p->K, p->a, p->gamma, p->max_trials, nullptr, 0));
+            LAUNCH(SUPCG_KIND_STV, st, enqueue_stv(w, st, p->K, p->a, p->gamma, p->max_trials, nullptr, 0));
             LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, 1, p->r, p->lambda, g->art_S, blocks, st));
         }
     }
@@ -1093,8 +1118,7 @@ static int enqueue_body(Workspace *w, const supcg_params *p, cudaStream_t st, in
     // previous norm pass) and by R d for the displacement d of S_TV, which S_TV writes in the
     // projector's layouts; the same sums as projecting x, in one pass over d
     if (p->perturb && p->K > 0) {                                               // steps 11-12
-        LAUNCH(SUPCG_KIND_STV, st, launch_stv(w->L(KT_STV, st), p->K, p->a, p->gamma, p->max_trials, nullptr,
-                                              want_snorm, dir));
+        LAUNCH(SUPCG_KIND_STV, st, enqueue_stv(w, st, p->K, p->a, p->gamma, p->max_trials, nullptr, want_snorm, dir));
         LAUNCH(SUPCG_KIND_FORWARD, st, launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 2, FWD_RUPD));
     } else {
         LAUNCH(SUPCG_KIND_VECTOR, st, launch_rupdate(w->L(KT_SINO, st)));
@@ -1178,7 +1202,7 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
         s0[c].muX = isnan(p->bayes_mu) ? 0.0 : p->bayes_mu;   // NaN: estimated from b below
         SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0[c], sizeof(Scal), cudaMemcpyHostToDevice, st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 2 * sizeof(unsigned), st));
+        SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.p, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.h, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
     }

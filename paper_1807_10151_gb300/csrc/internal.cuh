@@ -266,7 +266,7 @@ struct Prob {
     Scal *sc;
     double *partial;       // reduction partials (>= 2 * max blocks per kernel)
     unsigned *counter;     // last-block tickets [8]
-    unsigned *bar;         // cooperative barrier [2]: arrivals, generation
+    unsigned *bar;         // cooperative barriers: arrivals, generation; [2..3] a 64-bit count of arrivals (k_stv_tile)
     long long wait_limit;  // polls before a cooperative barrier gives up (supcg_set_wait_limit)
     int bar_extra;         // blocks a cooperative barrier waits for beyond its launch's (test hook, normally 0)
     double *log;           // nullable [max_iter][SUPCG_LOG_STRIDE]
@@ -668,6 +668,10 @@ int launch_stv(const Launch &L, int K, double a, double gamma, long long max_tri
                int want_snorm, const float *dir = nullptr);
 int launch_tv_tbar(const Launch &L);
 int stv_max_blocks_per_sm(int *out);
+int stv_tiles(int nx, int ny, int ti);          // blocks of k_stv_tile for an image, tiles of ti x 32 pixels
+int stv_tile_max_blocks(int ti, int *out);      // co-resident blocks of k_stv_tile
+int launch_stv_tile(const Launch &L, int ti, int K, double a, double gamma, long long max_trials, int *trials_out,
+                    int want_snorm);
 int cnn_forward(struct supcg_cnn_s *net, const float *d_x, const float *d_tbar, int count, cudaStream_t st);
 float *cnn_output(struct supcg_cnn_s *net);
 int cnn_shape(struct supcg_cnn_s *net, int *ny, int *nx);

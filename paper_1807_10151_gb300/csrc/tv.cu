@@ -10,7 +10,9 @@
 // data-dependent backtracking loop (repeat ... until TV(y~) <= TV(y)) runs
 // on the device without returning to the host.  Every block sums the
 // per-block FP64 partials in the same order, so all blocks take the same
-// accept / reject decision.
+// accept / reject decision.  Two kernels: k_stv_tile keeps the image in shared
+// memory through the K steps (images that fit, up to about 1100^2), k_stv walks
+// it in memory (larger images, and the learned direction's step).
 #include "internal.cuh"
 
 namespace supcg {
@@ -45,6 +47,13 @@ __device__ __forceinline__ Nb7 nb7_load(const float *__restrict__ y, int ld, int
     return v;
 }
 
+// The root of a TV term with differences a (down) and b (right).  Where the two differences are near the
+// rounding of the image a step's direction hangs on the last bit of this root, so it is pinned: one product
+// rounded, the other inside the FMA, which of the two as the kernels have always had it (root in a pixel's
+// own term and in the term of the pixel above it, root_b in that of the pixel left of it).
+__device__ __forceinline__ float root(float a, float b) { return sqrtf(__fmaf_rn(a, a, __fmul_rn(b, b))); }
+__device__ __forceinline__ float root_b(float a, float b) { return sqrtf(__fmaf_rn(b, b, __fmul_rn(a, a))); }
+
 // tbar at pixel (i, j) from its seven values; *Tb receives the root of the TV term
 // whose base is (i, j) (0 if that term does not exist).
 __device__ __forceinline__ float tbar_from(const Nb7 &v, int ny, int nx, int i, int j, float *Tb)
@@ -57,7 +66,7 @@ __device__ __forceinline__ float tbar_from(const Nb7 &v, int ny, int nx, int i, 
         const float a = yc - v.d, b = yc - v.r;
         if (a == 0.0f && b == 0.0f) undef = true;
         else {
-            const float T = sqrtf(a * a + b * b);
+            const float T = root(a, b);
             tb = T;
             g += (a + b) / T;
         }
@@ -66,13 +75,13 @@ __device__ __forceinline__ float tbar_from(const Nb7 &v, int ny, int nx, int i, 
         const float yu = v.u;
         const float a = yu - yc, b = yu - v.ur;
         if (a == 0.0f && b == 0.0f) undef = true;
-        else g -= a / sqrtf(a * a + b * b);
+        else g -= a / root(a, b);
     }
     if (j >= 1 && i + 1 < ny) {
         const float yl = v.l;
         const float a = yl - v.ld, b = yl - yc;
         if (a == 0.0f && b == 0.0f) undef = true;
-        else g -= b / sqrtf(a * a + b * b);
+        else g -= b / root_b(a, b);
     }
     *Tb = tb;
     return undef ? 0.0f : -g;
@@ -556,6 +565,456 @@ __global__ void __launch_bounds__(kTvThreads, 3) k_stv(const Prob *__restrict__ 
     // d, unless the last step wrote it (after the last barrier every block sees the final x);
     // no step ran when the plain loop had none (K = 0), and then no barrier either
     if (ok && !d_done) write_d(false, plain && K == 0, 0.0f);
+}
+
+// ------------------------------------------------------------ S_TV on resident tiles
+// S_TV with every problem's image held on the chip, a tile of TI x 32 pixels per block:
+// one grid barrier per trial.  In memory (k_stv) a step took three barriers with a pass
+// over the image each, 20 us at 512^2, of which the arithmetic is about one; what counts
+// is the number of barriers and of L2 round trips between them.  Here a trial forms
+// y~ = y + c tbar itself (the pair (x, xlo), as the accepted step does) and, before the
+// barrier that sums TV(y~), also tbar(y~) and its norm: if y~ is accepted, the next step
+// starts at once.
+//   A block holds y on its tile and one ring around it, and tbar of y there (its own
+// pixels' and one ring pixel's per thread, in registers), so it has y~ on both and
+// TV(y~), tbar(y~) on the tile.  tbar(y~) of the ring comes from the neighbours: each
+// block publishes its outermost rows and columns before the barrier and reads the ring
+// after it, together with the partial sums.  A ring pixel of y~ is computed by two
+// blocks, from the same values in the same order, bit for bit alike.  The published
+// values alternate between two buffers (z and g, free until the next gradient), since a
+// block may still be reading one trial's while another writes the next one's.  x is
+// written only at the end.
+//   A TV term's roots and quotients are computed once, at its base pixel, and meet the
+// pixels below and to the right of it in shared memory.  The values are those of
+// k_stv bit for bit, and so are the steps, as long as the two kernels' sums round to
+// the same FP32 step length.
+// Measured, K = 40 at 512^2 (one call): 867 -> 364 us, 6.6 us per step; a grid barrier is
+// about 1.4 us of it, the FP64 sum over the blocks' partials 1 us.
+constexpr int kStvThreads = 512, kStvWarps = kStvThreads / 32;
+
+template <int TI>
+struct StvTile {
+    static constexpr int H = TI + 2, W = 34, LD = 35;       // the tile and its ring; odd pitch
+    static constexpr int PX = TI / kStvWarps;               // pixels per thread
+    static constexpr int RING = 2 * W + 2 * TI;             // pixels of the ring
+    static_assert(RING <= kStvThreads - 64, "one ring pixel per thread, the first two warps left out");
+    float hi[2][H * LD], lo[2][H * LD];                     // y and y~ (high and low parts), in turn
+    float qa[H * LD], qb[H * LD];                           // a / T and b / T of the TV term based at the pixel
+};
+constexpr float kUndef = 4.0f;   // qa, qb of a term whose differences are both 0 (|a / T| <= 1 otherwise)
+
+// Pixel k of the ring around the tile, in the coordinates of the held region.
+template <int TI>
+__device__ __forceinline__ void stv_ring(int k, int &i, int &j)
+{
+    using S = StvTile<TI>;
+    if (k < S::W) { i = 0; j = k; return; }
+    k -= S::W;
+    if (k < S::W) { i = TI + 1; j = k; return; }
+    k -= S::W;
+    i = 1 + (k >> 1);
+    j = (k & 1) ? S::W - 1 : 0;
+}
+
+// x / T for y = 1 / T correctly rounded: Markstein's quotient (IBM J. Res. Dev. 34, 1990), correctly rounded
+// as the division itself is where x - q T is a normal number or 0.
+__device__ __forceinline__ float quotient(float x, float T, float y)
+{
+    const float q = __fmul_rn(x, y);
+    return __fmaf_rn(__fmaf_rn(-q, T, x), y, q);
+}
+
+// Grid barrier of the tile kernel: a counter of arrivals that only grows (`target` arrivals complete this
+// barrier).  One release by thread 0 covers the block's writes (the block barrier before it orders them),
+// and the acquiring poll the reads after it.  Bounded: false after `limit` polls.
+__device__ __forceinline__ bool stv_barrier(unsigned long long *ctr, unsigned long long target, long long limit, int *status,
+                                            int *sh_flag)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(ctr) : "memory");
+        int ok = 1;
+        long long it = 0;
+        for (;;) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+            if (v >= target) break;
+            if (++it > limit) {
+                ok = 0;
+                atomicExch(status, (int)SUPCG_ERR_TIMEOUT);
+                break;
+            }
+        }
+        *sh_flag = ok;
+    }
+    __syncthreads();
+    return *sh_flag;
+}
+
+// The step scalars of one thread.  An FP64 instruction holds the SM's FP64 pipe for about 38 cycles per warp
+// that issues it; inlined, these were turned into predicated code that every warp issued (350 FP64
+// instructions per step and block, the pipe 85 % busy: 456 us for 40 steps at 512^2 against 364).
+struct StvScalars {
+    double apow, gap;   // a^l (Scal::apow), gamma a^l
+    float gh, gl;       // gamma a^l as two FP32 parts
+};
+__device__ __noinline__ void stv_set_pow(StvScalars *s, double apow, double gamma)
+{
+    s->apow = apow;
+    s->gap = gamma * apow;
+    s->gh = (float)s->gap;
+    s->gl = (float)(s->gap - (double)s->gh);
+}
+// gamma a^l / sqrt(nn) rounded to FP32 (0 for nn = 0): on the FP32 pipe to about 2^-46 before the last
+// rounding, in FP64 outside its range.
+__device__ __noinline__ float stv_step(const StvScalars *s, double nn)
+{
+    if (!(nn > 0.0)) return 0.0f;
+    const float nh = (float)nn, gh = s->gh;
+    if (!(nh > 1e-30f && nh < 1e30f && gh > 1e-25f && gh < 1e25f)) return (float)(s->gap * rsqrt_fp64(nn));
+    const float nl = (float)(nn - (double)nh);
+    const float y = rsqrtf(nh);
+    const df m = df_mul(df{nh, nl}, df_prod(y, y));
+    const float e = __fsub_rn(__fsub_rn(1.0f, m.h), m.l);                          // 1 - nn y^2
+    const float yl = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, 0.5f * e));   // 1 / sqrt(nn) = y + yl
+    const df p = df_prod(gh, y);
+    return __fadd_rn(p.h, __fadd_rn(p.l, __fmaf_rn(gh, yl, __fmul_rn(s->gl, y))));
+}
+__device__ __noinline__ void stv_first_pow(StvScalars *s, const Scal *sc, double a, double gamma)
+{
+    const bool carried = sc->apow_ok && sc->apow_ell == sc->ell && sc->apow_a == a;
+    stv_set_pow(s, carried ? sc->apow : pow(a, (double)sc->ell), gamma);
+}
+__device__ __noinline__ void stv_next_pow(StvScalars *s, double a, double gamma) { stv_set_pow(s, s->apow * a, gamma); }
+// u <= v for sums of roots (>= 0, or NaN: false), on the integer pipe.
+__device__ __forceinline__ bool sum_le(double u, double v)
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(u), b = (unsigned long long)__double_as_longlong(v);
+    return a <= b && a <= 0x7FF0000000000000ull;
+}
+
+template <int TI>
+__global__ void __launch_bounds__(kStvThreads, 2) k_stv_tile(const Prob *__restrict__ probs, const int *__restrict__ prefix,
+                                                             int count, int K_arg, double a_arg, double gamma_arg,
+                                                             long long max_trials, int *trials_out, int want_snorm)
+{
+    using S = StvTile<TI>;
+    constexpr int LD = S::LD, PX = S::PX;
+    extern __shared__ __align__(16) unsigned char stv_raw[];
+    S &sm = *reinterpret_cast<S *>(stv_raw);
+    __shared__ __align__(16) double red[40];
+    __shared__ double sh_tot[2];
+    __shared__ float sh_c;
+    __shared__ int flag;
+    int local;
+    const int pi = find_problem(prefix, count, blockIdx.x, &local);
+    const Prob &P = probs[pi];
+    Scal *sc = P.sc;
+    if (sc->done) return;
+    const int K = P.stv_own ? P.stv_K : K_arg;
+    const double a = P.stv_own ? P.stv_a : a_arg, gamma = P.stv_own ? P.stv_gamma : gamma_arg;
+    const int nb = prefix[pi + 1] - prefix[pi];
+    const int nx = P.nx, ny = P.ny, ld = P.nxp;
+    const int tiles_j = (nx + 31) / 32;
+    const int ti = local / tiles_j, i0 = ti * TI, j0 = (local - ti * tiles_j) * 32;
+    const int t = threadIdx.x, tx = t & 31, ty = t >> 5, lane = tx;
+    const bool has_lo = P.xlo != nullptr;
+    // the step scalars live in the first thread of the last warp, whose FP64 work runs beside the other warps'
+    const bool scalars = t == kStvThreads - 32;
+    unsigned long long *ctr = reinterpret_cast<unsigned long long *>(P.bar + 2);
+    const unsigned long long per = (unsigned long long)(nb + P.bar_extra);
+    unsigned long long target = 0;   // thread 0's: arrivals before this launch's first barrier, then the next barrier's
+    if (t == 0) {
+        // (this block has not arrived yet, so the barrier under way is this launch's first)
+        unsigned long long v;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+        target = v / per * per;
+    }
+    long long ell = sc->ell;
+    __shared__ StvScalars sh_sc;
+    if (scalars) stv_first_pow(&sh_sc, sc, a, gamma);
+    // y on the tile and its ring (0 off the image: no formula below uses it)
+    int cur = 0;
+    for (int e = t; e < S::H * S::W; e += kStvThreads) {
+        const int ri = e / S::W, rj = e - ri * S::W, i = i0 + ri - 1, j = j0 + rj - 1;
+        const bool in = i >= 0 && i < ny && j >= 0 && j < nx;
+        const size_t p = in ? (size_t)i * ld + j : 0;
+        sm.hi[0][ri * LD + rj] = in ? P.x[p] : 0.0f;
+        sm.lo[0][ri * LD + rj] = (in && has_lo) ? P.xlo[p] : 0.0f;
+    }
+    // this thread's ring pixel
+    int rk = 0;
+    size_t rp = 0;
+    bool ring = false;
+    if (t >= 64 && t - 64 < S::RING) {
+        int ri, rj;
+        stv_ring<TI>(t - 64, ri, rj);
+        const int i = i0 + ri - 1, j = j0 + rj - 1;
+        rk = ri * LD + rj;
+        ring = i >= 0 && i < ny && j >= 0 && j < nx;
+        if (ring) rp = (size_t)i * ld + j;
+    }
+    __syncthreads();
+    // The tile's part of TV and (want_t) of ||tbar||^2 of buffer y, tbar into tn and its outermost rows and
+    // columns published; the block's sums into its partial of `slot`.
+    float tn[PX];
+    auto tile_sums = [&](const float *y, bool want_t, int slot) {
+        df d_tv = df_make(0.0f), d_nn = df_make(0.0f);
+        float qs[PX];   // (a + b) / T of the own terms
+        // a term's root, and its quotients into qa, qb
+        auto term = [&](int q, bool exists, float *sum_q) {
+            float T = 0.0f, va = 0.0f, vb = 0.0f, vs = 0.0f;
+            if (exists) {
+                const float yc = y[q], a1 = yc - y[q + LD], b1 = yc - y[q + 1];
+                if (a1 == 0.0f && b1 == 0.0f) {
+                    va = vb = vs = kUndef;
+                } else {
+                    const float Tl = root_b(a1, b1);
+                    T = root(a1, b1);
+                    const float iv = __frcp_rn(T);
+                    va = quotient(a1, T, iv);
+                    vb = quotient(b1, Tl, __frcp_rn(Tl));
+                    vs = quotient(__fadd_rn(a1, b1), T, iv);
+                }
+            }
+            sm.qa[q] = va;
+            sm.qb[q] = vb;
+            *sum_q = vs;
+            return T;
+        };
+        if (want_t) {
+#pragma unroll
+            for (int q = 0; q < PX; ++q) {
+                const int r = ty + kStvWarps * q, i = i0 + r, j = j0 + tx;
+                df_acc(d_tv, term((r + 1) * LD + tx + 1, i + 1 < ny && j + 1 < nx, &qs[q]));
+            }
+            if (t < 32 + TI) {   // the terms based above the tile and left of it
+                const int ri = t < 32 ? 0 : t - 31, rj = t < 32 ? t + 1 : 0, i = i0 + ri - 1, j = j0 + rj - 1;
+                float s;
+                (void)term(ri * LD + rj, i >= 0 && j >= 0 && i + 1 < ny && j + 1 < nx, &s);
+            }
+            __syncthreads();
+            float *pub = slot ? P.g : P.z;
+#pragma unroll
+            for (int q = 0; q < PX; ++q) {
+                const int r = ty + kStvWarps * q, i = i0 + r, j = j0 + tx;
+                const float up = sm.qa[r * LD + tx + 1], le = sm.qb[(r + 1) * LD + tx];
+                const bool undef = qs[q] == kUndef || up == kUndef || le == kUndef;
+                const float g = __fsub_rn(__fsub_rn(qs[q], up), le);
+                tn[q] = (undef || i >= ny || j >= nx) ? 0.0f : -g;
+                df_acc_prod(d_nn, tn[q], tn[q]);
+                if (i < ny && j < nx && (r == 0 || r == TI - 1 || tx == 0 || tx == 31)) pub[(size_t)i * ld + j] = tn[q];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < PX; ++q) {
+                const int r = ty + kStvWarps * q, e = (r + 1) * LD + tx + 1;
+                if (i0 + r + 1 < ny && j0 + tx + 1 < nx) {
+                    const float a1 = y[e] - y[e + LD], b1 = y[e] - y[e + 1];
+                    df_acc(d_tv, root(a1, b1));
+                }
+            }
+        }
+        double b1, b2;
+        block_sum_df2<kStvThreads>(d_tv, d_nn, red, &b1, &b2);
+        if (t == 0) reinterpret_cast<double2 *>(P.partial)[(size_t)slot * nb + local] = make_double2(b1, b2);
+    };
+    // the sums of all blocks, in the same order in each: TV by warp 0, ||tbar||^2 by warp 1 (an FP64 add holds
+    // a quarter of the SM's narrow FP64 pipe for many cycles, so the two chains run on different quarters)
+    auto totals = [&](int slot) {
+        const double *pp = P.partial + (size_t)slot * 2 * nb + ty;
+        double v = 0.0;
+        for (int b = lane; b < nb; b += 32 * 8) {
+            double u[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u[k] = b + 32 * k < nb ? __ldcg(pp + 2 * (b + 32 * k)) : 0.0;
+            v += ((u[0] + u[1]) + (u[2] + u[3])) + ((u[4] + u[5]) + (u[6] + u[7]));
+        }
+        v = warp_sum(v);
+        if (lane == 0) sh_tot[ty] = v;
+    };
+    // the barrier after tile_sums, then the totals; tbar of the ring pixel meanwhile
+    float rt = 0.0f, rn = 0.0f;   // tbar of this thread's ring pixel: of y, of y~
+    auto meet = [&](int slot, bool want_t) {
+        target += per;
+        if (!stv_barrier(ctr, target, P.wait_limit, &sc->status, &flag)) return false;
+        if (ty < 2) totals(slot);
+        else if (want_t && ring) rn = __ldcg((slot ? P.g : P.z) + rp);
+        __syncthreads();
+        return true;
+    };
+    int slot = 0;
+    bool ok = true, timed_out = false;
+    long long total_trials = 0;
+    float c = 0.0f, tc[PX];       // tc: tbar of y on the tile
+    tile_sums(sm.hi[0], true, slot);
+    if (!meet(slot, true)) return;
+    const double tv_first = sh_tot[0];
+    double tv_y = tv_first, tv_half = 0.0;   // TV of y; of the last accepted y~
+    for (int step = 0; step < K && ok; ++step) {
+        // y is the last accepted image (buffer cur), its tbar in tn and rn, TV and ||tbar||^2 in sh_tot
+        const float *yh = sm.hi[cur], *yl = sm.lo[cur];
+        float *zh = sm.hi[cur ^ 1], *zl = sm.lo[cur ^ 1];
+#pragma unroll
+        for (int q = 0; q < PX; ++q) tc[q] = tn[q];
+        rt = rn;
+        const double nn = sh_tot[1];
+        const bool last = step == K - 1;
+        long long trials = 0;
+        for (;;) {
+            if (trials >= max_trials) {
+                if (local == 0 && t == 0) atomicExch(&sc->status, (int)SUPCG_ERR_BACKTRACK);
+                ok = false;
+                break;
+            }
+            if (scalars) sh_c = stv_step(&sh_sc, nn);   // gamma a^l / ||tbar||
+            __syncthreads();
+            c = sh_c;   // y~ = y + c tbar
+            ++ell;
+            ++trials;
+            if (scalars) stv_next_pow(&sh_sc, a, gamma);   // for the next trial: a^(l + 1)
+            auto move = [&](int q, float tq) {
+                if (has_lo) {
+                    const df v = df_add(df{yh[q], yl[q]}, df_prod(c, tq));
+                    zh[q] = v.h;
+                    zl[q] = v.l;
+                } else {
+                    zh[q] = __fmaf_rn(c, tq, yh[q]);
+                }
+            };
+#pragma unroll
+            for (int q = 0; q < PX; ++q) move((ty + kStvWarps * q + 1) * LD + tx + 1, tc[q]);
+            if (ring) move(rk, rt);
+            __syncthreads();
+            slot ^= 1;
+            tile_sums(zh, !last, slot);
+            if (!meet(slot, !last)) {
+                ok = false;
+                timed_out = true;
+                break;
+            }
+            if (sum_le(sh_tot[0], tv_y)) break;   // until TV(y~) <= TV(y); else y and its tbar stay
+        }
+        total_trials += trials;
+        if (!ok) break;
+        if (trials_out && local == 0 && t == 0) trials_out[(size_t)pi * K + step] = (int)trials;
+        cur ^= 1;
+        tv_y = tv_half = sh_tot[0];
+    }
+    const float *yh = sm.hi[cur], *yl = sm.lo[cur];
+    __syncthreads();
+    // ||s_k||^2 for the log, from the image before the steps (still in x)
+    double sn = 0.0;
+    if (ok && want_snorm) {
+        double s = 0.0;
+#pragma unroll
+        for (int q = 0; q < PX; ++q) {
+            const int r = ty + kStvWarps * q, i = i0 + r, j = j0 + tx;
+            if (i < ny && j < nx) {
+                const size_t p = (size_t)i * ld + j;
+                const int e = (r + 1) * LD + tx + 1;
+                const double dlt = ((double)yh[e] - (double)P.x[p]) + (has_lo ? (double)yl[e] - (double)P.xlo[p] : 0.0);
+                s += dlt * dlt;
+            }
+        }
+        s = block_sum<kStvThreads>(s, red);
+        slot ^= 1;
+        if (t == 0) reinterpret_cast<double2 *>(P.partial)[(size_t)slot * nb + local] = make_double2(s, 0.0);
+        timed_out = !meet(slot, false);
+        ok = !timed_out;
+        sn = sh_tot[0];
+    }
+    if (local == 0 && scalars) {
+        sc->ell = ell;
+        sc->apow = sh_sc.apow;
+        sc->apow_a = a;
+        sc->apow_ell = ell;
+        sc->apow_ok = 1;
+        sc->trials = total_trials;
+        sc->tv_k = tv_first;
+        sc->tv_half = tv_half;
+        sc->snorm2 = sn;
+    }
+    if (timed_out) return;
+    // x and, after K steps, the displacement d in the projector's layouts; with one plain step d is c tbar
+    // itself (the low part of x would not show in it), else the difference from the image before the steps
+    const bool plain1 = K == 1 && !want_snorm;
+    float *tr = sm.qa;   // the transpose of d, TI x 33
+    float dv[PX];
+#pragma unroll
+    for (int q = 0; q < PX; ++q) {
+        const int r = ty + kStvWarps * q, i = i0 + r, j = j0 + tx;
+        dv[q] = 0.0f;
+        if (i < ny && j < nx) {
+            const size_t p = (size_t)i * ld + j;
+            const int e = (r + 1) * LD + tx + 1;
+            if (plain1) dv[q] = __fmul_rn(c, tc[q]);
+            else dv[q] = __fadd_rn(__fsub_rn(yh[e], P.x[p]), has_lo ? __fsub_rn(yl[e], P.xlo[p]) : 0.0f);
+            P.x[p] = yh[e];
+            if (has_lo) P.xlo[p] = yl[e];
+            if (ok) {
+                P.d[p] = dv[q];
+                if (P.dm) P.dm[(size_t)i * ld + (nx - 1 - j)] = dv[q];
+            }
+        }
+    }
+    if (!ok) return;
+#pragma unroll
+    for (int q = 0; q < PX; ++q) tr[(ty + kStvWarps * q) * 33 + tx] = dv[q];
+    __syncthreads();
+    for (int e = t; e < 32 * TI; e += kStvThreads) {   // consecutive threads on consecutive rows of the image
+        const int cc = e / TI, r = e - cc * TI;
+        const int i = i0 + r, j = j0 + cc;
+        if (i < ny && j < nx) {
+            P.dT[(size_t)j * P.nyp + i] = tr[r * 33 + cc];
+            if (P.dmT) P.dmT[(size_t)(nx - 1 - j) * P.nyp + i] = tr[r * 33 + cc];
+        }
+    }
+}
+
+int stv_tiles(int nx, int ny, int ti) { return ((ny + ti - 1) / ti) * ((nx + 31) / 32); }
+
+template <int TI>
+static int stv_tile_blocks_t(int *out)
+{
+    int rc = func_attrs_once((const void *)k_stv_tile<TI>, (int)sizeof(StvTile<TI>), (int)cudaSharedmemCarveoutMaxShared);
+    if (rc) return rc;
+    int dev = 0, nsm = 0, per_sm = 0;
+    SUPCG_CUDA_TRY(cudaGetDevice(&dev));
+    SUPCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stv_tile<TI>, kStvThreads, sizeof(StvTile<TI>)));
+    *out = nsm * per_sm;
+    return SUPCG_OK;
+}
+int stv_tile_max_blocks(int ti, int *out)
+{
+    return ti == 32 ? stv_tile_blocks_t<32>(out) : (ti == 64 ? stv_tile_blocks_t<64>(out) : stv_tile_blocks_t<128>(out));
+}
+
+template <int TI>
+static int launch_stv_tile_t(const Launch &L, int K, double a, double gamma, long long max_trials, int *trials_out,
+                             int want_snorm)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(L.blocks);
+    cfg.blockDim = dim3(kStvThreads);
+    cfg.dynamicSmemBytes = sizeof(StvTile<TI>);
+    cfg.stream = L.st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SUPCG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_stv_tile<TI>, L.probs, L.prefix, L.count, K, a, gamma, max_trials, trials_out,
+                                      want_snorm));
+    return SUPCG_OK;
+}
+int launch_stv_tile(const Launch &L, int ti, int K, double a, double gamma, long long max_trials, int *trials_out,
+                    int want_snorm)
+{
+    if (ti == 32) return launch_stv_tile_t<32>(L, K, a, gamma, max_trials, trials_out, want_snorm);
+    if (ti == 64) return launch_stv_tile_t<64>(L, K, a, gamma, max_trials, trials_out, want_snorm);
+    return launch_stv_tile_t<128>(L, K, a, gamma, max_trials, trials_out, want_snorm);
 }
 
 int stv_max_blocks_per_sm(int *out)
