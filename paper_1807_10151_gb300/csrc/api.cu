@@ -671,7 +671,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         auto al = [](size_t b) { return (b + 255) / 256 * 256; };
         const size_t sizes[] = {img * 4, imgT * 4, img * 4, imgT * 4, img * 4, img * 4, img * 4, img * 4,
                                 sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, sizeof(Scal),
-                                npart * 8, 16 * 4, 4 * 4, (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 8,
+                                npart * 8, 16 * 4, 8 * 4, (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 8,
                                 2 * (size_t)g->bparts * img * 8,
                                 (size_t)std::max(nb[KT_BWD][c], nb[KT_BWD2][c]) * 4, img * 4, img * 4,
                                 mir * img * 4, mir * imgT * 4, mir * img * 4, mir * imgT * 4,
@@ -956,7 +956,7 @@ extern "C" int supcg_superiorize(supcg_geometry g, float *d_x, double a, double 
     Scal s0 = {};
     s0.ell = *h_ell;
     SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
+    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
     if ((rc = launch_stage_in(w->L(KT_TR, st), 0))) return rc;
     if ((rc = enqueue_stv(w, st, K, a, gamma, max_trials, K > 0 ? w->trials_dev : nullptr, 0))) return rc;
     if ((rc = launch_store_out(w->L(KT_VEC, st), 0))) return rc;
@@ -1046,23 +1046,24 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
     Scal s0 = {};
     s0.muX = isnan(p->mu) ? 0.0 : p->mu;
     SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
+    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
     SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st), 1));   // b -> bpad
     if (isnan(p->mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
-    const int init_blocks = (int)std::min<size_t>(8192, (m + 1) / 2);
+    const int init_blocks = (int)std::min<size_t>(8192, (m + 63) / 64);
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_art_init(w->dp, p->r, init_blocks, st));   // norms, u = 0, x = mu_X
     int cap = 0;
-    if ((rc = art_max_blocks(&cap))) return rc;
+    const int side = std::max(g->nx, g->ny);
+    if ((rc = art_max_blocks(side, &cap))) return rc;
     const int rays = (g->U + g->art_S - 1) / g->art_S;   // rays per class, one block each
     const int blocks = std::max(1, std::min(cap, rays));
     if (p->K == 0) {
         if (p->cycles > 0)
-            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, p->cycles, p->r, p->lambda, g->art_S, blocks, st));
+            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, side, p->cycles, p->r, p->lambda, g->art_S, blocks, st));
     } else {
         for (int c = 0; c < p->cycles; ++c) {   // SupART: S_TV, then one cycle
             LAUNCH(SUPCG_KIND_STV, st, enqueue_stv(w, st, p->K, p->a, p->gamma, p->max_trials, nullptr, 0));
-            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, 1, p->r, p->lambda, g->art_S, blocks, st));
+            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, side, 1, p->r, p->lambda, g->art_S, blocks, st));
         }
     }
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_store_out(w->L(KT_VEC, st), 0));
@@ -1202,7 +1203,7 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
         s0[c].muX = isnan(p->bayes_mu) ? 0.0 : p->bayes_mu;   // NaN: estimated from b below
         SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0[c], sizeof(Scal), cudaMemcpyHostToDevice, st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 4 * sizeof(unsigned), st));
+        SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.p, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
         SUPCG_CUDA_TRY(cudaMemsetAsync(P.h, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
     }

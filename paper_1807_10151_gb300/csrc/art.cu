@@ -14,17 +14,14 @@
 // (bounded) separates consecutive classes.  A ray's entries are the
 // projectors' (the same exact-split delta and trapezoid), evaluated once for
 // the ray sum <R_i, x> (a Kahan-compensated FP32 sum per thread, the
-// threads' sums added in FP64) and again for the update (FP32 FMA; this
-// part's FP64 pipe is narrow).  One block per ray: its threads take a few
-// rows each and issue all their loads before using them (the pixels sit in
-// L2, and a long chain of dependent loads had dominated).
+// threads' pairs added in double-float arithmetic) and again for the update
+// (FP32 FMA).  One block per ray: its threads take a few rows each.
 #include "internal.cuh"
 
 namespace supcg {
 
-constexpr int kArtThreads = 64;      // k_art_init: two warps, one ray each
-constexpr int kArtRayThreads = 128;  // k_art: one block per ray of a class
-constexpr int kArtRows = 4;          // rows per thread per group: their 4 x 3 loads issued together
+constexpr int kArtThreads = 64;      // k_art_init: one ray per thread
+constexpr int kArtRayThreads = 256;  // k_art: one block per ray of a class
 
 // The per-ray constants of a ray's entries (the projectors' exact split).
 struct ArtRay {
@@ -77,40 +74,31 @@ __device__ __forceinline__ void art_row(const Prob &P, const ViewP &vp, const Ar
     }
 }
 
-// f(pixel offset, unit weight) for every entry of ray (vp, u) with a nonzero
-// weight, over the rows lane, lane + 32, ... (used where latency does not matter).
-template <typename F>
-__device__ __forceinline__ void art_ray(const Prob &P, const ViewP &vp, int u, int lane, F &&f)
-{
-    const ArtRay R = art_ray_setup(P, vp, u);
-    for (int o = R.lo + lane; o <= R.hi; o += 32) {
-        int pix[3];
-        float w[3];
-        art_row(P, vp, R, o, pix, w);
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            if (w[k] != 0.0f) f(pix[k], w[k]);
-    }
-}
-
 // 1 / (1 + r^2 ||R_i||^2) for every ray (FP64), u = 0, and x = mu_X on the image
-// (the starting point of the method).  One warp per ray, grid-stride.
+// (the starting point of the method).  One ray per thread (no pixel is read, so neither
+// the rows' order nor their spread over lanes matters), its squares summed in double-float
+// arithmetic: with a warp per ray and FP64 squares the narrow FP64 pipe held this at
+// 2.35 ms for the 522000 rays of 512^2 / 720 views, 0.60 ms now.
 __global__ void __launch_bounds__(kArtThreads) k_art_init(const Prob *__restrict__ probs, double r)
 {
     const Prob &P = probs[0];
-    const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * (kArtThreads / 32) + (threadIdx.x >> 5), W = gridDim.x * (kArtThreads / 32);
-    for (int i = gw; i < P.V * P.U; i += W) {
-        const int v = i / P.U, u = i - v * P.U;
+    const long long rays = (long long)P.V * P.U;
+    for (long long i = (long long)blockIdx.x * kArtThreads + threadIdx.x; i < rays; i += (long long)gridDim.x * kArtThreads) {
+        const int v = (int)(i / P.U), u = (int)(i - (long long)v * P.U);
         const ViewP vp = P.views[v];
-        double s = 0.0;
-        art_ray(P, vp, u, lane, [&](int, float w) { s += (double)w * (double)w; });
-        s = warp_sum(s);
-        if (lane == 0) {
-            const double pl = (double)vp.P;
-            P.art_rn[i] = 1.0 / (1.0 + r * r * pl * pl * s);
-            P.art_u[i] = 0.0;
+        const ArtRay R = art_ray_setup(P, vp, u);
+        df s = df_make(0.0f);
+        for (int o = R.lo; o <= R.hi; ++o) {
+            int pix[3];
+            float w[3];
+            art_row(P, vp, R, o, pix, w);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (w[k] != 0.0f) df_acc_prod(s, w[k], w[k]);
         }
+        const double pl = (double)vp.P;
+        P.art_rn[i] = 1.0 / (1.0 + r * r * pl * pl * df_to_double(s));
+        P.art_u[i] = 0.0;
     }
     const float mu = (float)P.sc->muX;
     const size_t n = (size_t)P.ny * P.nxp;
@@ -120,14 +108,33 @@ __global__ void __launch_bounds__(kArtThreads) k_art_init(const Prob *__restrict
     }
 }
 
-// `cycles` full ART cycles on P.x (one cooperative launch; every block takes
-// part in every class barrier).  Block b takes the rays u = c + S (b + k nblocks)
-// of class c; its threads split the ray's rows, kArtRows at a time, and load
-// the rows' candidates before using them (the pixels were written by other
-// blocks before the last barrier: read past L1).
+// The step of one ray: c from its sum s (in units of the plateau length pl), u <- u + c; returns r c pl.
+// A call, not inlined: an FP64 instruction holds the SM's pipe for tens of cycles per warp that issues it, and
+// inlined under a test for one thread it may be issued, predicated off, by all.
+__device__ __noinline__ float art_coef(df s, float pl, float b, double ui, double rn, double r, double lam, double *u)
+{
+    const double cc = lam * (r * ((double)b - (double)pl * df_to_double(s)) - ui) * rn;
+    *u = ui + cc;
+    return (float)(r * cc * (double)pl);
+}
+
+// `cycles` full ART cycles on P.x (one cooperative launch; every block takes part in every
+// class barrier).  Block b takes the rays u = c + S (b + k nblocks) of class c.  The classes
+// are a serial chain (1440 per cycle at 512^2 / 720 views), so what counts is the time from
+// one barrier to the next: the first ROWS rows per thread of the block's next ray, their
+// weights and its scalars are evaluated between the arrival at a barrier and the wait, so
+// that after it only the pixels are read, summed and updated.  The pixels are read through
+// L1 (the barrier's fence empties it of what other blocks have written since): a row's two or
+// three candidates are neighbours, and past L1 each of them fetched its own sector from L2.
+// A class takes 4.4 us, 6.6 before (the weights after the barrier, the threads' sums added in
+// FP64, 128 threads per ray); of it about 2.5 us are the barrier and the SMs with three
+// of the 363 blocks are the last to arrive.  Rows beyond the first
+// ROWS * kArtRayThreads, and further rays of a block, are evaluated where they are used.
+template <int ROWS>
 __global__ void __launch_bounds__(kArtRayThreads) k_art(const Prob *__restrict__ probs, int cycles, double r,
                                                         double lam, int S)
 {
+    constexpr int N = 3 * ROWS, GROUP = ROWS * kArtRayThreads;
     __shared__ int flag;
     __shared__ __align__(16) double red[40];
     __shared__ float sh_rc;
@@ -135,99 +142,128 @@ __global__ void __launch_bounds__(kArtRayThreads) k_art(const Prob *__restrict__
     Scal *sc = P.sc;
     const int t = threadIdx.x;
     float *x = P.x;
+    GridCount bar(P.bar + 4, gridDim.x + P.bar_extra);
+
+    // the pixels and weights of rows o0, o0 + kArtRayThreads, ... of a ray
+    auto rows_of = [&](const ViewP &vp, const ArtRay &R, int o0, int *pix, float *w) {
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+            const int o = o0 + q * kArtRayThreads;
+            if (o <= R.hi) {
+                art_row(P, vp, R, o, pix + 3 * q, w + 3 * q);
+            } else {
+                w[3 * q] = w[3 * q + 1] = w[3 * q + 2] = 0.0f;
+                pix[3 * q] = pix[3 * q + 1] = pix[3 * q + 2] = 0;
+            }
+        }
+    };
+    // the ray under way: its first group's pixels and weights, thread 0's scalars
+    int gpix[N];
+    float gw[N], bi = 0.0f, pl = 0.0f;
+    double ui = 0.0, rni = 0.0;
+    bool more = false;   // rows beyond the first group
+    auto prepare = [&](int v, int u) {
+        const ViewP vp = P.views[v];
+        const ArtRay R = art_ray_setup(P, vp, u);
+        rows_of(vp, R, R.lo + t, gpix, gw);
+        more = R.hi - R.lo >= GROUP;
+        pl = vp.P;
+        if (t == 0) {
+            bi = P.bpad[(size_t)v * P.Up + u];
+            ui = P.art_u[(size_t)v * P.U + u];   // (written only by this block, at the ray's last visit)
+            rni = P.art_rn[(size_t)v * P.U + u];
+        }
+    };
+    float ks, kc;   // Kahan pair of the thread's terms of <R_i, x>
+    auto load_and_sum = [&](const int *pix, const float *w, float *xv) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) xv[k] = (w[k] != 0.0f) ? x[pix[k]] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const float y = __fmaf_rn(w[k], xv[k], -kc);
+            const float tt = __fadd_rn(ks, y);
+            kc = __fsub_rn(__fsub_rn(tt, ks), y);
+            ks = tt;
+        }
+    };
+    auto visit = [&](int v, int u) {
+        float gx[N];   // (the class's other rays touch none of these pixels: still current at the update)
+        ks = kc = 0.0f;
+        load_and_sum(gpix, gw, gx);
+        if (more) {
+            const ViewP vp = P.views[v];
+            const ArtRay R = art_ray_setup(P, vp, u);
+            for (int o0 = R.lo + t + GROUP; o0 <= R.hi; o0 += GROUP) {
+                int pix[N];
+                float w[N], xv[N];
+                rows_of(vp, R, o0, pix, w);
+                load_and_sum(pix, w, xv);
+            }
+        }
+        const df s = block_sum_pair<kArtRayThreads>(df{ks, -kc}, red);   // in thread 0
+        if (t == 0) sh_rc = art_coef(s, pl, bi, ui, rni, r, lam, P.art_u + (size_t)v * P.U + u);
+        __syncthreads();
+        const float rcf = sh_rc;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (gw[k] != 0.0f) x[gpix[k]] = __fmaf_rn(rcf, gw[k], gx[k]);
+        if (more) {
+            const ViewP vp = P.views[v];
+            const ArtRay R = art_ray_setup(P, vp, u);
+            for (int o0 = R.lo + t + GROUP; o0 <= R.hi; o0 += GROUP) {
+                int pix[N];
+                float w[N], xv[N];
+                rows_of(vp, R, o0, pix, w);
+#pragma unroll
+                for (int k = 0; k < N; ++k) xv[k] = (w[k] != 0.0f) ? x[pix[k]] : 0.0f;
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    if (w[k] != 0.0f) x[pix[k]] = __fmaf_rn(rcf, w[k], xv[k]);
+            }
+        }
+    };
+    const int u0 = S * blockIdx.x;   // the block's first ray of a class: c + u0
+    if (u0 < P.U) prepare(0, u0);
     for (int cyc = 0; cyc < cycles; ++cyc) {
         for (int v = 0; v < P.V; ++v) {
-            const ViewP vp = P.views[v];
             for (int c = 0; c < S; ++c) {
-                for (int u = c + S * blockIdx.x; u < P.U; u += S * gridDim.x) {   // block-uniform
-                    const ArtRay R = art_ray_setup(P, vp, u);
-                    const size_t i = (size_t)v * P.U + u;
-                    double bi = 0.0, ui = 0.0, rni = 0.0;   // the ray's scalars, fetched while the sum runs
-                    if (t == 0) {
-                        bi = (double)P.bpad[(size_t)v * P.Up + u];
-                        ui = P.art_u[i];
-                        rni = P.art_rn[i];
+                if (c + u0 < P.U) {
+                    visit(v, c + u0);
+                    for (int u = c + u0 + S * gridDim.x; u < P.U; u += S * gridDim.x) {   // block-uniform
+                        prepare(v, u);
+                        __syncthreads();   // sh_rc and red are reused
+                        visit(v, u);
                     }
-                    float ks = 0.0f, kc = 0.0f;   // Kahan pair of the thread's terms of <R_i, x>
-                    // a ray of at most kArtRows x kArtRayThreads rows: each thread's rows, weights and
-                    // pixel values are gathered once and kept for the update (the class's other rays
-                    // touch none of these pixels, so the values are still current then)
-                    const bool one_group = R.hi - R.lo < kArtRows * kArtRayThreads;
-                    int gpix[3 * kArtRows];
-                    float gw[3 * kArtRows], gx[3 * kArtRows];
-                    for (int o0 = R.lo + t; o0 <= R.hi; o0 += kArtRows * kArtRayThreads) {
-                        int *pix = gpix;
-                        float *w = gw, *xv = gx;
-#pragma unroll
-                        for (int q = 0; q < kArtRows; ++q) {
-                            const int o = o0 + q * kArtRayThreads;
-                            if (o <= R.hi) {
-                                art_row(P, vp, R, o, pix + 3 * q, w + 3 * q);
-                            } else {
-                                w[3 * q] = w[3 * q + 1] = w[3 * q + 2] = 0.0f;
-                                pix[3 * q] = pix[3 * q + 1] = pix[3 * q + 2] = 0;
-                            }
-                        }
-#pragma unroll
-                        for (int k = 0; k < 3 * kArtRows; ++k) xv[k] = (w[k] != 0.0f) ? __ldcg(x + pix[k]) : 0.0f;
-#pragma unroll
-                        for (int k = 0; k < 3 * kArtRows; ++k) {
-                            const float y = __fmaf_rn(w[k], xv[k], -kc);
-                            const float tt = __fadd_rn(ks, y);
-                            kc = __fsub_rn(__fsub_rn(tt, ks), y);
-                            ks = tt;
-                        }
-                    }
-                    const double s = block_sum<kArtRayThreads>((double)ks - (double)kc, red);   // in thread 0
-                    if (t == 0) {
-                        const double cc = lam * (r * (bi - (double)vp.P * s) - ui) * rni;
-                        P.art_u[i] = ui + cc;
-                        sh_rc = (float)(r * cc * (double)vp.P);
-                    }
-                    __syncthreads();
-                    const float rcf = sh_rc;
-                    if (one_group) {
-                        if (t <= R.hi - R.lo) {   // (threads past the ray's rows gathered nothing)
-#pragma unroll
-                            for (int k = 0; k < 3 * kArtRows; ++k)
-                                if (gw[k] != 0.0f) x[gpix[k]] = __fmaf_rn(rcf, gw[k], gx[k]);
-                        }
-                    } else
-                    for (int o0 = R.lo + t; o0 <= R.hi; o0 += kArtRows * kArtRayThreads) {
-                        int pix[3 * kArtRows];
-                        float w[3 * kArtRows], xv[3 * kArtRows];
-#pragma unroll
-                        for (int q = 0; q < kArtRows; ++q) {
-                            const int o = o0 + q * kArtRayThreads;
-                            if (o <= R.hi) {
-                                art_row(P, vp, R, o, pix + 3 * q, w + 3 * q);
-                            } else {
-                                w[3 * q] = w[3 * q + 1] = w[3 * q + 2] = 0.0f;
-                                pix[3 * q] = pix[3 * q + 1] = pix[3 * q + 2] = 0;
-                            }
-                        }
-#pragma unroll
-                        for (int k = 0; k < 3 * kArtRows; ++k) xv[k] = (w[k] != 0.0f) ? __ldcg(x + pix[k]) : 0.0f;
-#pragma unroll
-                        for (int k = 0; k < 3 * kArtRows; ++k)
-                            if (w[k] != 0.0f) x[pix[k]] = __fmaf_rn(rcf, w[k], xv[k]);
-                    }
-                    __syncthreads();   // sh_rc and red are reused by the block's next ray
                 }
-                if (!coop_barrier(P.bar, gridDim.x + P.bar_extra, &sc->status, &flag, P.wait_limit)) return;   // bounded: SUPCG_ERR_TIMEOUT
+                bar.arrive();
+                const int nc = c + 1 < S ? c + 1 : 0, nv = nc ? v : (v + 1 < P.V ? v + 1 : 0);
+                if (nc + u0 < P.U) prepare(nv, nc + u0);
+                if (!bar.wait<true>(P.wait_limit, &sc->status, &flag)) return;   // bounded: SUPCG_ERR_TIMEOUT
             }
         }
     }
 }
 
-int art_max_blocks(int *out)
+// Rows per thread: enough for the longest ray in one group, up to 4 (images up to 1024 rows and columns).
+template <typename F>
+static int with_art_rows(int side, F &&f)
+{
+    if (side <= kArtRayThreads) return f(k_art<1>);
+    if (side <= 2 * kArtRayThreads) return f(k_art<2>);
+    return f(k_art<4>);
+}
+
+int art_max_blocks(int side, int *out)
 {
     int nsm = 0, per_sm = 0, dev = 0;
     SUPCG_CUDA_TRY(cudaGetDevice(&dev));
     SUPCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_art, kArtRayThreads, 0));
+    const int rc = with_art_rows(side, [&](auto *kernel) -> int {
+        SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kArtRayThreads, 0));
+        return SUPCG_OK;
+    });
     *out = nsm * per_sm;
-    return SUPCG_OK;
+    return rc;
 }
 
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st)
@@ -237,7 +273,7 @@ int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st)
     return SUPCG_OK;
 }
 
-int launch_art(const Prob *d_prob, int cycles, double r, double lam, int S, int blocks, cudaStream_t st)
+int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
@@ -249,8 +285,10 @@ int launch_art(const Prob *d_prob, int cycles, double r, double lam, int S, int 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SUPCG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_art, d_prob, cycles, r, lam, S));
-    return SUPCG_OK;
+    return with_art_rows(side, [&](auto *kernel) -> int {
+        SUPCG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, d_prob, cycles, r, lam, S));
+        return SUPCG_OK;
+    });
 }
 
 } // namespace supcg

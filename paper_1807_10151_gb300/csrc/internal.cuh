@@ -266,7 +266,8 @@ struct Prob {
     Scal *sc;
     double *partial;       // reduction partials (>= 2 * max blocks per kernel)
     unsigned *counter;     // last-block tickets [8]
-    unsigned *bar;         // cooperative barriers: arrivals, generation; [2..3] a 64-bit count of arrivals (k_stv_tile)
+    unsigned *bar;         // cooperative barriers: arrivals, generation (k_stv); 64-bit counts of arrivals (GridCount):
+                           // [2..3] k_stv_tile, [4..5] k_art (a count belongs to one number of blocks)
     long long wait_limit;  // polls before a cooperative barrier gives up (supcg_set_wait_limit)
     int bar_extra;         // blocks a cooperative barrier waits for beyond its launch's (test hook, normally 0)
     double *log;           // nullable [max_iter][SUPCG_LOG_STRIDE]
@@ -379,21 +380,26 @@ __device__ __forceinline__ df warp_sum_df(df v)
     return v;
 }
 template <int NT>
-__device__ __forceinline__ double block_sum_df(df v, double *sh)
+__device__ __forceinline__ df block_sum_pair(df v, double *sh)
 {
     float2 *s2 = reinterpret_cast<float2 *>(sh);
     v = warp_sum_df(v);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0) s2[w] = make_float2(v.h, v.l);
     __syncthreads();
-    double r = 0.0;
+    df u = {0.0f, 0.0f};
     if (w == 0) {
-        df u = (l < NT / 32) ? df{s2[l].x, s2[l].y} : df{0.0f, 0.0f};
+        if (l < NT / 32) u = df{s2[l].x, s2[l].y};
         u = warp_sum_df(u);
-        if (l == 0) r = df_to_double(u);
     }
     __syncthreads();
-    return r;
+    return u;
+}
+template <int NT>
+__device__ __forceinline__ double block_sum_df(df v, double *sh)
+{
+    const df u = block_sum_pair<NT>(v, sh);
+    return threadIdx.x == 0 ? df_to_double(u) : 0.0;
 }
 
 // Two block sums in one pass (one sweep of shuffles, one shared-memory round): the
@@ -558,6 +564,59 @@ __device__ __forceinline__ bool coop_barrier(unsigned *bar, unsigned nblocks, in
     return *sh_flag;
 }
 
+// Grid barriers among the co-resident blocks of a cooperative launch by a counter of arrivals that only grows:
+// `blocks` arrivals complete a barrier.  Thread 0's release covers the block's writes (the block barrier before
+// it orders them), its poll the block's later reads; one L2 round trip each, where coop_barrier makes three (the
+// generation, the arrival, the release).  Every block arrives at every barrier; between arrive and
+// wait it may do what needs no other block.  A counter belongs to one kernel and number of blocks, so that it is
+// a multiple of that number when a launch begins.
+struct GridCount {
+    unsigned long long *ctr;
+    unsigned long long per, target;   // thread 0's: the arrivals that complete the barrier under way
+    __device__ GridCount(unsigned *words, int blocks)
+        : ctr(reinterpret_cast<unsigned long long *>(words)), per((unsigned long long)blocks), target(0)
+    {
+        if (threadIdx.x == 0) {   // (this block has not arrived yet, so the barrier under way is the launch's first)
+            unsigned long long v;
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+            target = v / per * per;
+        }
+    }
+    __device__ __forceinline__ void arrive()
+    {
+        __syncthreads();
+        target += per;
+        if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(ctr) : "memory");
+    }
+    // Bounded: false after `limit` polls (and raises SUPCG_ERR_TIMEOUT in *status); the same in every thread.
+    // L1: the block then reads through L1 what other blocks wrote.  The polls are relaxed and one fence follows
+    // them (an acquiring poll empties the SM's L1 each time); without it the last poll acquires, which is sooner
+    // done (364 against 379 us for 40 steps of k_stv_tile at 512^2).
+    template <bool L1>
+    __device__ __forceinline__ bool wait(long long limit, int *status, int *sh_flag)
+    {
+        if (threadIdx.x == 0) {
+            int ok = 1;
+            long long it = 0;
+            for (;;) {
+                unsigned long long v;
+                if (L1) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+                else asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+                if (v >= target) break;
+                if (++it > limit) {
+                    ok = 0;
+                    atomicExch(status, (int)SUPCG_ERR_TIMEOUT);
+                    break;
+                }
+            }
+            if (L1) __threadfence();
+            *sh_flag = ok;
+        }
+        __syncthreads();
+        return *sh_flag;
+    }
+};
+
 // ----------------------------------------------------------------- TMA / mbarrier
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -646,9 +705,9 @@ struct Launch {
 int launch_forward(const Launch &L, const Launch &La, int which, int mode);   // La: every view's items
 int launch_backward(const Launch &L, int mode, int bwin);
 int launch_backward2(const Launch &L, int bwin);   // g from r and h from q in one pass
-int art_max_blocks(int *out);                                           // co-resident blocks of k_art
+int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side the longer one of the image
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st);
-int launch_art(const Prob *d_prob, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
+int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
 int backward_blocks(int nx, int ny, int dual, int parts);
 int encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims,
                  const cuuint64_t *strides_bytes, const cuuint32_t *box);

@@ -624,33 +624,6 @@ __device__ __forceinline__ float quotient(float x, float T, float y)
     return __fmaf_rn(__fmaf_rn(-q, T, x), y, q);
 }
 
-// Grid barrier of the tile kernel: a counter of arrivals that only grows (`target` arrivals complete this
-// barrier).  One release by thread 0 covers the block's writes (the block barrier before it orders them),
-// and the acquiring poll the reads after it.  Bounded: false after `limit` polls.
-__device__ __forceinline__ bool stv_barrier(unsigned long long *ctr, unsigned long long target, long long limit, int *status,
-                                            int *sh_flag)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(ctr) : "memory");
-        int ok = 1;
-        long long it = 0;
-        for (;;) {
-            unsigned long long v;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
-            if (v >= target) break;
-            if (++it > limit) {
-                ok = 0;
-                atomicExch(status, (int)SUPCG_ERR_TIMEOUT);
-                break;
-            }
-        }
-        *sh_flag = ok;
-    }
-    __syncthreads();
-    return *sh_flag;
-}
-
 // The step scalars of one thread.  An FP64 instruction holds the SM's FP64 pipe for about 38 cycles per warp
 // that issues it; inlined, these were turned into predicated code that every warp issued (350 FP64
 // instructions per step and block, the pipe 85 % busy: 456 us for 40 steps at 512^2 against 364).
@@ -721,15 +694,7 @@ __global__ void __launch_bounds__(kStvThreads, 2) k_stv_tile(const Prob *__restr
     const bool has_lo = P.xlo != nullptr;
     // the step scalars live in the first thread of the last warp, whose FP64 work runs beside the other warps'
     const bool scalars = t == kStvThreads - 32;
-    unsigned long long *ctr = reinterpret_cast<unsigned long long *>(P.bar + 2);
-    const unsigned long long per = (unsigned long long)(nb + P.bar_extra);
-    unsigned long long target = 0;   // thread 0's: arrivals before this launch's first barrier, then the next barrier's
-    if (t == 0) {
-        // (this block has not arrived yet, so the barrier under way is this launch's first)
-        unsigned long long v;
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
-        target = v / per * per;
-    }
+    GridCount bar(P.bar + 2, nb + P.bar_extra);
     long long ell = sc->ell;
     __shared__ StvScalars sh_sc;
     if (scalars) stv_first_pow(&sh_sc, sc, a, gamma);
@@ -836,8 +801,8 @@ __global__ void __launch_bounds__(kStvThreads, 2) k_stv_tile(const Prob *__restr
     // the barrier after tile_sums, then the totals; tbar of the ring pixel meanwhile
     float rt = 0.0f, rn = 0.0f;   // tbar of this thread's ring pixel: of y, of y~
     auto meet = [&](int slot, bool want_t) {
-        target += per;
-        if (!stv_barrier(ctr, target, P.wait_limit, &sc->status, &flag)) return false;
+        bar.arrive();
+        if (!bar.wait<false>(P.wait_limit, &sc->status, &flag)) return false;
         if (ty < 2) totals(slot);
         else if (want_t && ring) rn = __ldcg((slot ? P.g : P.z) + rp);
         __syncthreads();
