@@ -97,6 +97,7 @@ struct Workspace {
     int bparts = 0;             // view parts of every problem's backprojector, 0 if they differ
     int mirror = 0;             // 1: some problem has mirror pairs of views
     int stv_ti = 0;             // rows of k_stv_tile's tiles; 0: the images do not fit, S_TV walks them in memory
+    bool wc_ready = false;      // the problems' frequency tables are filled
     std::vector<void *> allocs;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t body_exec = nullptr;
@@ -675,7 +676,8 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
                                 2 * (size_t)g->bparts * img * 8,
                                 (size_t)std::max(nb[KT_BWD][c], nb[KT_BWD2][c]) * 4, img * 4, img * 4,
                                 mir * img * 4, mir * imgT * 4, mir * img * 4, mir * imgT * 4,
-                                img * 4, imgT * 4, mir * img * 4, mir * imgT * 4, sino * 8, sino * 8};
+                                img * 4, imgT * 4, mir * img * 4, mir * imgT * 4, sino * 8, sino * 8,
+                                (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 16};
         constexpr int kPieces = sizeof(sizes) / sizeof(sizes[0]);
         size_t total = 0;
         for (size_t s : sizes) total += al(s);
@@ -706,6 +708,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.dmT = mir ? (float *)ptrs[28] : nullptr;
         P.rd = (double *)ptrs[29];
         P.qd = (double *)ptrs[30];
+        P.wc = (double2 *)ptrs[31];
         if (mir) w->mirror = 1;
         P.border = g->dborder;
         P.border_all = g->dborder_all;
@@ -815,6 +818,17 @@ static int ops_ws(supcg_geometry g, int batch, Workspace **out)
     return SUPCG_OK;
 }
 
+// The preconditioner's filter: the workspace's table of frequencies on its first use, then D from mu and rho.
+static int enqueue_filter(Workspace *w, cudaStream_t st)
+{
+    if (!w->wc_ready) {
+        const int rc = launch_fft_wc(w->L(KT_VEC, st));
+        if (rc) return rc;
+        w->wc_ready = true;
+    }
+    return launch_fft_dtab(w->L(KT_VEC, st));
+}
+
 static size_t elem_size(int storage) { return storage == SUPCG_BF16 ? 2 : 4; }
 
 // ------------------------------------------------------------------ operators
@@ -887,7 +901,7 @@ extern "C" int supcg_precondition(supcg_geometry g, double mu, double rho, const
     for (int b = 0; b < batch; ++b) w->hp[b].storage = g->storage;
     if (rc) return rc;
     if ((rc = launch_stage_in(w->L(KT_TR, st), 1))) return rc;
-    if ((rc = launch_fft_dtab(w->L(KT_VEC, st)))) return rc;
+    if ((rc = enqueue_filter(w, st))) return rc;
     if ((rc = enqueue_precond(w, st, 1))) return rc;
     return launch_store_out(w->L(KT_VEC, st), 2);
 }
@@ -1210,7 +1224,7 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_in(w->L(KT_TR, st), 0));
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st), 1));
     if (p->bayes_r > 0.0 && isnan(p->bayes_mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
-    if (p->precondition) LAUNCH(SUPCG_KIND_VECTOR, st, launch_fft_dtab(w->L(KT_VEC, st)));
+    if (p->precondition) LAUNCH(SUPCG_KIND_VECTOR, st, enqueue_filter(w, st));
     if ((rc = enqueue_init(w, p, st))) return rc;
 
     const int want_snorm = d_log != nullptr;
