@@ -81,6 +81,7 @@ static int fft_factor(int n, int *rad)
 } // namespace supcg
 
 // ------------------------------------------------------------------ objects
+constexpr int kInlineTrials = 64;   // S_TV trial counts read back together with the scalars
 enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWD2, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
 
 struct Workspace {
@@ -88,7 +89,10 @@ struct Workspace {
     std::vector<supcg_geometry> geoms;
     std::vector<unsigned> versions;   // the geometries' layout versions when this was built
     std::vector<Prob> hp;
+    std::vector<Prob> on_device;      // what dp holds (empty: nothing yet)
     Prob *dp = nullptr;
+    Scal *scals = nullptr;            // device (behind dprefix): the problems' scalars, then kInlineTrials ints
+    cudaEvent_t last = nullptr;       // end of the last standalone operator's work
     int *dprefix = nullptr;     // KT_COUNT x (count + 1)
     int blocks[KT_COUNT] = {};
     int smem_rows = 0, smem_cols = 0;
@@ -129,6 +133,7 @@ struct Workspace {
         if (cap_stream) cudaStreamDestroy(cap_stream);
         for (void *p : allocs) cudaFree(p);
         if (dp) cudaFree(dp);
+        if (last) cudaEventDestroy(last);
         if (dprefix) cudaFree(dprefix);
         if (trials_dev) cudaFree(trials_dev);
         if (lstage) cudaFree(lstage);
@@ -654,10 +659,16 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         hprefix[kt * (w->count + 1) + w->count] = acc;
         w->blocks[kt] = acc;
     }
-    if (cudaMalloc(&w->dprefix, sizeof(int) * hprefix.size()) != cudaSuccess ||
+    // the prefix tables, then the problems' scalars and the inline trial counts
+    const size_t prefix_bytes = (sizeof(int) * hprefix.size() + 255) / 256 * 256;
+    const size_t scal_bytes = sizeof(Scal) * w->count + kInlineTrials * sizeof(int);
+    if (cudaMalloc(&w->dprefix, prefix_bytes + scal_bytes) != cudaSuccess) { delete w; return SUPCG_ERR_NOMEM; }
+    w->scals = reinterpret_cast<Scal *>(reinterpret_cast<char *>(w->dprefix) + prefix_bytes);
+    if (cudaMemset(w->scals, 0, scal_bytes) != cudaSuccess ||
+        cudaEventCreateWithFlags(&w->last, cudaEventDisableTiming) != cudaSuccess ||
         cudaMemcpy(w->dprefix, hprefix.data(), sizeof(int) * hprefix.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         delete w;
-        return SUPCG_ERR_NOMEM;
+        return SUPCG_ERR_CUDA;
     }
 
     // buffers: one allocation per problem, 256-byte aligned pieces
@@ -671,7 +682,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         const size_t npart = std::max<size_t>(std::max(12 * (size_t)nb[KT_STV][c], 4 * (size_t)nb[KT_STVT][c]), 2 * (size_t)maxblk) + 64;
         auto al = [](size_t b) { return (b + 255) / 256 * 256; };
         const size_t sizes[] = {img * 4, imgT * 4, img * 4, imgT * 4, img * 4, img * 4, img * 4, img * 4,
-                                sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, sizeof(Scal),
+                                sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, 0,
                                 npart * 8, 16 * 4, 8 * 4, (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 8,
                                 2 * (size_t)g->bparts * img * 8,
                                 (size_t)std::max(nb[KT_BWD][c], nb[KT_BWD2][c]) * 4, img * 4, img * 4,
@@ -691,7 +702,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.x = (float *)ptrs[0]; P.xT = (float *)ptrs[1]; P.p = (float *)ptrs[2]; P.pT = (float *)ptrs[3];
         P.g = (float *)ptrs[4]; P.z = (float *)ptrs[5]; P.h = (float *)ptrs[6]; P.tbar = (float *)ptrs[7];
         P.r = (float *)ptrs[8]; P.q = (float *)ptrs[9]; P.bpad = (float *)ptrs[10];
-        P.C = (double2 *)ptrs[11]; P.sc = (Scal *)ptrs[12]; P.partial = (double *)ptrs[13];
+        P.C = (double2 *)ptrs[11]; P.sc = w->scals + c; P.partial = (double *)ptrs[13];
         P.counter = (unsigned *)ptrs[14]; P.bar = (unsigned *)ptrs[15]; P.Dtab = (float2 *)ptrs[16];
         P.bsplit = (float2 *)ptrs[17]; P.tilecnt = (unsigned *)ptrs[18]; P.xlo = (float *)ptrs[19];
         P.bparts = g->bparts;
@@ -722,7 +733,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         w->bw_max = std::max(w->bw_max, g->BW);
         P.views = g->dviews; P.vlist = g->dvlist;
         P.fx = g->fx; P.fy = g->fy;
-        P.storage = g->storage;
+        P.storage = SUPCG_F32;   // (a solve's; the operators pass the geometry's)
         P.stv_blocks = nb[KT_STV][c];
         P.mu = 1e-5; P.rho = 0.8; P.precond = 1;
         P.r2 = 0.0;
@@ -784,17 +795,44 @@ static bool batch_ws_current(supcg_geometry owner, const std::vector<supcg_geome
     return true;
 }
 
+// The descriptors on the device, copied again only when they changed since the last copy (the caller's arrays of
+// a standalone operator are kernel arguments, so calls in a row change nothing).
 static int ws_upload(Workspace *w, cudaStream_t st)
 {
     for (Prob &P : w->hp) {
         P.wait_limit = g_wait_limit.load();
         P.bar_extra = g_bar_extra.load();
     }
-    // synchronous copy from pageable memory: safe to modify hp afterwards
+    if (w->on_device.size() == w->hp.size() &&
+        !memcmp(w->on_device.data(), w->hp.data(), sizeof(Prob) * w->hp.size()))
+        return SUPCG_OK;
+    // synchronous copy from pageable memory, after the work that reads the old ones: safe to modify hp afterwards
+    w->on_device.clear();
     SUPCG_CUDA_TRY(cudaStreamSynchronize(st));
     SUPCG_CUDA_TRY(cudaMemcpy(w->dp, w->hp.data(), sizeof(Prob) * w->count, cudaMemcpyHostToDevice));
+    w->on_device = w->hp;
     return SUPCG_OK;
 }
+
+// A standalone operator's work on the workspace: after the last such call's, whatever stream that was on (the
+// scratch is shared), with the descriptors up to date; its end is marked when the call returns.
+struct OpsScope {
+    Workspace *w;
+    cudaStream_t st;
+    int rc = SUPCG_OK;
+    OpsScope(Workspace *ws, cudaStream_t stream) : w(ws), st(stream)
+    {
+        if (cudaStreamWaitEvent(st, w->last, 0) != cudaSuccess) {
+            (void)cudaGetLastError();
+            rc = SUPCG_ERR_CUDA;
+        } else {
+            rc = ws_upload(w, st);
+        }
+    }
+    ~OpsScope() { (void)cudaEventRecord(w->last, st); }
+    OpsScope(const OpsScope &) = delete;
+    OpsScope &operator=(const OpsScope &) = delete;
+};
 
 // S_TV over the problems of w: on resident tiles where they fit and no learned direction is given.
 static int enqueue_stv(Workspace *w, cudaStream_t st, int K, double a, double gamma, long long max_trials, int *trials_out,
@@ -832,6 +870,12 @@ static int enqueue_filter(Workspace *w, cudaStream_t st)
 static size_t elem_size(int storage) { return storage == SUPCG_BF16 ? 2 : 4; }
 
 // ------------------------------------------------------------------ operators
+static Io batch_io(const void *in, void *out, size_t in_elems, size_t out_elems, int storage)
+{
+    const size_t es = elem_size(storage);
+    return Io{(const char *)in, (char *)out, in_elems * es, out_elems * es, storage};
+}
+
 extern "C" int supcg_project(supcg_geometry g, const void *d_x, void *d_y, int batch, void *stream)
 {
     if (!g || !d_x || !d_y || batch < 1) return SUPCG_ERR_ARG;
@@ -839,14 +883,11 @@ extern "C" int supcg_project(supcg_geometry g, const void *d_x, void *d_y, int b
     int rc = ops_ws(g, batch, &w);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t es = elem_size(g->storage);
-    for (int b = 0; b < batch; ++b) {
-        w->hp[b].in_user = (const char *)d_x + (size_t)b * g->nx * g->ny * es;
-        w->hp[b].out_user = (char *)d_y + (size_t)b * g->V * g->U * es;
-    }
-    if ((rc = ws_upload(w, st))) return rc;
-    if ((rc = launch_stage_in(w->L(KT_TR, st), 0))) return rc;
-    return launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_PLAIN);
+    const Io io = batch_io(d_x, d_y, (size_t)g->nx * g->ny, (size_t)g->V * g->U, g->storage);
+    OpsScope scope(w, st);
+    if (scope.rc) return scope.rc;
+    if ((rc = launch_stage_in(w->L(KT_TR, st), io))) return rc;
+    return launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_PLAIN, io);
 }
 
 extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, int batch, void *stream)
@@ -856,28 +897,22 @@ extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, i
     int rc = ops_ws(g, batch, &w);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t es = elem_size(g->storage);
-    for (int b = 0; b < batch; ++b) {
-        w->hp[b].in_user = (const char *)d_y + (size_t)b * g->V * g->U * es;
-        w->hp[b].out_user = (char *)d_x + (size_t)b * g->nx * g->ny * es;
-    }
-    if ((rc = ws_upload(w, st))) return rc;
-    if ((rc = launch_stage_sino(w->L(KT_SINO, st), 0))) return rc;
-    if ((rc = launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin))) return rc;
-    return launch_store_out(w->L(KT_VEC, st), 1);
+    const size_t m = (size_t)g->V * g->U, n = (size_t)g->nx * g->ny, es = elem_size(g->storage);
+    const Io io = batch_io(d_y, d_x, m, n, g->storage);
+    OpsScope scope(w, st);
+    if (scope.rc) return scope.rc;
+    // straight into the caller's image, unless it overlaps the sinogram still being read
+    const char *y = (const char *)d_y, *x = (const char *)d_x;
+    if (y + batch * m * es <= x || x + batch * n * es <= y) return launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin, io);
+    Io to_g = io;
+    to_g.out = nullptr;
+    if ((rc = launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin, to_g))) return rc;
+    return launch_store_out(w->L(KT_VEC, st), 2, io);
 }
 
 static int check_precond(double mu, double rho)
 {
     return (!(rho > 0.5) || !(rho <= 1.0) || !(mu >= 0.0) || !isfinite(mu)) ? SUPCG_ERR_PRECOND : SUPCG_OK;
-}
-
-static int enqueue_precond(Workspace *w, cudaStream_t st, int standalone)
-{
-    int rc;
-    if ((rc = launch_fft_rows(w->L(KT_ROWS, st), 0, standalone, w->smem_rows))) return rc;
-    if ((rc = launch_fft_cols(w->L(KT_COLS, st), standalone, w->smem_cols))) return rc;
-    return launch_fft_rows(w->L(KT_ROWS, st), 1, standalone, w->smem_rows);
 }
 
 extern "C" int supcg_precondition(supcg_geometry g, double mu, double rho, const float *d_g, float *d_z, int batch,
@@ -889,21 +924,18 @@ extern "C" int supcg_precondition(supcg_geometry g, double mu, double rho, const
     Workspace *w;
     if ((rc = ops_ws(g, batch, &w))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    for (int b = 0; b < batch; ++b) {
-        Prob &P = w->hp[b];
-        P.in_user = d_g + (size_t)b * g->nx * g->ny;
-        P.out_user = d_z + (size_t)b * g->nx * g->ny;
+    for (Prob &P : w->hp) {
         P.mu = mu;
         P.rho = rho;
-        P.storage = SUPCG_F32;
     }
-    rc = ws_upload(w, st);
-    for (int b = 0; b < batch; ++b) w->hp[b].storage = g->storage;
-    if (rc) return rc;
-    if ((rc = launch_stage_in(w->L(KT_TR, st), 1))) return rc;
+    const size_t n = (size_t)g->nx * g->ny;
+    const Io io = batch_io(d_g, d_z, n, n, SUPCG_F32);   // (all of g is read before z is written: they may alias)
+    OpsScope scope(w, st);
+    if (scope.rc) return scope.rc;
     if ((rc = enqueue_filter(w, st))) return rc;
-    if ((rc = enqueue_precond(w, st, 1))) return rc;
-    return launch_store_out(w->L(KT_VEC, st), 2);
+    if ((rc = launch_fft_rows(w->L(KT_ROWS, st), 0, 1, w->smem_rows, io))) return rc;
+    if ((rc = launch_fft_cols(w->L(KT_COLS, st), 1, w->smem_cols))) return rc;
+    return launch_fft_rows(w->L(KT_ROWS, st), 1, 1, w->smem_rows, io);
 }
 
 static int read_scal(const Prob &P, Scal *h, cudaStream_t st)
@@ -920,18 +952,14 @@ extern "C" int supcg_tv_tbar(supcg_geometry g, const float *d_y, float *d_tbar, 
     int rc = ops_ws(g, 1, &w);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    Prob &P = w->hp[0];
-    P.in_user = d_y;
-    P.out_user = d_tbar;
-    P.storage = SUPCG_F32;
-    rc = ws_upload(w, st);
-    P.storage = g->storage;
-    if (rc) return rc;
-    if ((rc = launch_stage_in(w->L(KT_TR, st), 0))) return rc;
+    const Io io = batch_io(d_y, d_tbar, 0, 0, SUPCG_F32);
+    OpsScope scope(w, st);
+    if (scope.rc) return scope.rc;
+    if ((rc = launch_stage_in(w->L(KT_TR, st), io))) return rc;
     if ((rc = launch_tv_tbar(w->L(KT_TV, st)))) return rc;
-    if ((rc = launch_store_out(w->L(KT_VEC, st), 3))) return rc;
+    if ((rc = launch_store_out(w->L(KT_VEC, st), 1, io))) return rc;
     Scal s;
-    if ((rc = read_scal(P, &s, st))) return rc;
+    if ((rc = read_scal(w->hp[0], &s, st))) return rc;
     h_out[0] = s.tv_k;
     h_out[1] = s.snorm2;
     return SUPCG_OK;
@@ -953,32 +981,40 @@ extern "C" int supcg_superiorize(supcg_geometry g, float *d_x, double a, double 
     Workspace *w;
     if ((rc = ops_ws(g, 1, &w))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    Prob &P = w->hp[0];
-    P.in_user = d_x;
-    P.out_user = d_x;
-    P.storage = SUPCG_F32;
-    rc = ws_upload(w, st);
-    P.storage = g->storage;
-    if (rc) return rc;
-    if (K > w->trials_cap) {
-        if (w->trials_dev) cudaFree(w->trials_dev);
-        w->trials_dev = nullptr;
-        w->trials_cap = 0;
-        SUPCG_CUDA_TRY(cudaMalloc(&w->trials_dev, sizeof(int) * K));
-        w->trials_cap = K;
+    // trial counts: behind the scalars for a single copy back, in an array of their own for many steps
+    int *trials = reinterpret_cast<int *>(w->scals + w->count);
+    if (K > kInlineTrials) {
+        if (K > w->trials_cap) {
+            if (w->trials_dev) cudaFree(w->trials_dev);
+            w->trials_dev = nullptr;
+            w->trials_cap = 0;
+            SUPCG_CUDA_TRY(cudaMalloc(&w->trials_dev, sizeof(int) * K));
+            w->trials_cap = K;
+        }
+        trials = w->trials_dev;
     }
+    const Io io = batch_io(d_x, d_x, 0, 0, SUPCG_F32);
     Scal s0 = {};
     s0.ell = *h_ell;
-    SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
-    if ((rc = launch_stage_in(w->L(KT_TR, st), 0))) return rc;
-    if ((rc = enqueue_stv(w, st, K, a, gamma, max_trials, K > 0 ? w->trials_dev : nullptr, 0))) return rc;
-    if ((rc = launch_store_out(w->L(KT_VEC, st), 0))) return rc;
-    Scal s;
-    if ((rc = read_scal(P, &s, st))) return rc;
-    if (h_trials && K > 0) SUPCG_CUDA_TRY(cudaMemcpy(h_trials, w->trials_dev, sizeof(int) * K, cudaMemcpyDeviceToHost));
-    *h_ell = s.ell;
-    return s.status;
+    OpsScope scope(w, st);
+    if (scope.rc) return scope.rc;
+    if ((rc = launch_init(w->L(KT_VEC, st), s0))) return rc;
+    if ((rc = launch_stage_in(w->L(KT_TR, st), io))) return rc;
+    if ((rc = enqueue_stv(w, st, K, a, gamma, max_trials, K > 0 ? trials : nullptr, 0))) return rc;
+    if ((rc = launch_store_out(w->L(KT_VEC, st), 0, io))) return rc;
+    struct {
+        Scal s;
+        int trials[kInlineTrials];
+    } h;
+    static_assert(sizeof(h) == sizeof(Scal) + kInlineTrials * sizeof(int), "the trial counts follow the scalars");
+    SUPCG_CUDA_TRY(cudaMemcpyAsync(&h, w->scals, sizeof(h), cudaMemcpyDeviceToHost, st));
+    SUPCG_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h_trials && K > 0) {
+        if (K <= kInlineTrials) memcpy(h_trials, h.trials, sizeof(int) * K);
+        else SUPCG_CUDA_TRY(cudaMemcpy(h_trials, trials, sizeof(int) * K, cudaMemcpyDeviceToHost));
+    }
+    *h_ell = h.s.ell;
+    return h.s.status;
 }
 
 // ------------------------------------------------------------------ launch accounting
@@ -1045,24 +1081,19 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
     if (!g->art_u) SUPCG_CUDA_TRY(cudaMalloc(&g->art_u, sizeof(double) * m));
     if (!g->art_rn) SUPCG_CUDA_TRY(cudaMalloc(&g->art_rn, sizeof(double) * m));
     Prob &P = w->hp[0];
-    P.in_user = d_x;
-    P.out_user = d_x;
     P.in_user2 = d_b;
     P.art_u = g->art_u;
     P.art_rn = g->art_rn;
-    P.storage = SUPCG_F32;
     float *xlo = P.xlo;
     P.xlo = nullptr;   // ART's row actions and SupART's S_TV work on the FP32 image alone
-    rc = ws_upload(w, st);
-    P.storage = g->storage;
+    OpsScope scope(w, st);
     P.xlo = xlo;
-    if (rc) return rc;
+    if (scope.rc) return scope.rc;
+    const Io io = batch_io(d_x, d_x, 0, 0, SUPCG_F32);
     Scal s0 = {};
     s0.muX = isnan(p->mu) ? 0.0 : p->mu;
-    SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0, sizeof(Scal), cudaMemcpyHostToDevice, st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
-    SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
-    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st), 1));   // b -> bpad
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_init(w->L(KT_VEC, st), s0));
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st)));      // b -> bpad
     if (isnan(p->mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
     const int init_blocks = (int)std::min<size_t>(8192, (m + 63) / 64);
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_art_init(w->dp, p->r, init_blocks, st));   // norms, u = 0, x = mu_X
@@ -1080,7 +1111,7 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
             LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, side, 1, p->r, p->lambda, g->art_S, blocks, st));
         }
     }
-    LAUNCH(SUPCG_KIND_VECTOR, st, launch_store_out(w->L(KT_VEC, st), 0));
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_store_out(w->L(KT_VEC, st), 0, io));
     Scal s;
     if ((rc = read_scal(P, &s, st))) return rc;
     rep->cycles = s.status ? 0 : p->cycles;
@@ -1197,7 +1228,6 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
         P.stv_gamma = q.gamma;
         P.precond = p->precondition ? 1 : 0;
         P.r2 = p->bayes_r > 0.0 ? p->bayes_r * p->bayes_r : 0.0;
-        P.storage = SUPCG_F32;
         P.log = (c == 0) ? d_log : nullptr;
         P.trace = (c == 0) ? d_trace : nullptr;
         P.se_ref = (se && se->ref) ? se->ref : nullptr;
@@ -1206,23 +1236,14 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
         P.se_ay = se ? se->ay * P.ny : 0.0;
     }
     rc = ws_upload(w, st);
-    for (int c = 0; c < w->count; ++c) w->hp[c].storage = w->geoms[c]->storage;
     if (rc) return rc;
-    std::vector<Scal> s0(w->count);
-    for (int c = 0; c < w->count; ++c) {
-        const Prob &P = w->hp[c];
-        s0[c] = Scal();
-        s0[c].eps = p->eps;
-        s0[c].init = 1;
-        s0[c].muX = isnan(p->bayes_mu) ? 0.0 : p->bayes_mu;   // NaN: estimated from b below
-        SUPCG_CUDA_TRY(cudaMemcpyAsync(P.sc, &s0[c], sizeof(Scal), cudaMemcpyHostToDevice, st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.counter, 0, 16 * sizeof(unsigned), st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.bar, 0, 8 * sizeof(unsigned), st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.p, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
-        SUPCG_CUDA_TRY(cudaMemsetAsync(P.h, 0, sizeof(float) * (size_t)P.ny * P.nxp, st));
-    }
-    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_in(w->L(KT_TR, st), 0));
-    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st), 1));
+    Scal s0 = {};
+    s0.eps = p->eps;
+    s0.init = 1;
+    s0.muX = isnan(p->bayes_mu) ? 0.0 : p->bayes_mu;   // NaN: estimated from b below
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_init(w->L(KT_VEC, st), s0));
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_in(w->L(KT_TR, st)));
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st)));
     if (p->bayes_r > 0.0 && isnan(p->bayes_mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
     if (p->precondition) LAUNCH(SUPCG_KIND_VECTOR, st, enqueue_filter(w, st));
     if ((rc = enqueue_init(w, p, st))) return rc;
@@ -1276,8 +1297,7 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
     }
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_store_out(w->L(KT_VEC, st), 0));
     std::vector<Scal> hs(w->count);
-    for (int c = 0; c < w->count; ++c)
-        SUPCG_CUDA_TRY(cudaMemcpyAsync(&hs[c], w->hp[c].sc, sizeof(Scal), cudaMemcpyDeviceToHost, st));
+    SUPCG_CUDA_TRY(cudaMemcpyAsync(hs.data(), w->scals, sizeof(Scal) * w->count, cudaMemcpyDeviceToHost, st));
     SUPCG_CUDA_TRY(cudaStreamSynchronize(st));
     int worst = SUPCG_OK;
     for (int c = 0; c < w->count; ++c) {

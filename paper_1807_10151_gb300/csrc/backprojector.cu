@@ -103,14 +103,15 @@ __device__ __forceinline__ void bwd_view_x2(const ViewP &vp, float pb0, const ui
 }
 
 // R^T y over one sinogram (mode BWD_G: y = r into g, BWD_H: y = q into h,
-// BWD_PLAIN: y = the staged input into g), or, DUAL, over two in one pass:
+// BWD_PLAIN: the caller's sinogram into the caller's image, or into g where io has none), or, DUAL, over two in one pass:
 // g from r and h from q (h = A p for the beta of the next step of Algorithm 2,
 // deferred to this pass: alpha takes p^T A p from the forward projector's ||q||^2).
 // FIXED_PARTS: the view parts per tile when every problem of the launch has that
 // (default) number, so the part arithmetic is compile-time; 0: each problem's own.
 template <bool DUAL, int FIXED_PARTS>
 __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Prob *__restrict__ probs,
-                                                          const int *__restrict__ prefix, int count, int mode)
+                                                          const int *__restrict__ prefix, int count, int mode,
+                                                          Io io)
 {
     constexpr int NS = BwdShape<DUAL>::NS, TI = BwdShape<DUAL>::TI, PX = BwdShape<DUAL>::PX;
     // proj_dyn: [2][NS][kBwdViewChunk][bwin] sinogram windows
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
 
     const float *sino0 = (!DUAL && mode == BWD_H) ? P.q : P.r;
     const float *sino1 = P.q;
+    const void *user = io.in + (size_t)pi * io.in_step;
     const int Up = P.Up;
     // tile corners in pixel-centre coordinates
     const float Xa = __fsub_rn(__int2float_rn(j0), P.cx), Xb = __fsub_rn(__int2float_rn(j0 + kBwdTileJ - 1), P.cx);
@@ -210,7 +212,15 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
             float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
             const int ub = ulo_sh[buf][vv] + 4 * k4;
             if (v < P.V && ub >= 0 && ub + 3 < Up) {
-                val = __ldg(reinterpret_cast<const float4 *>((s ? sino1 : sino0) + (size_t)v * Up + ub));
+                if (!DUAL && mode == BWD_PLAIN) {   // the caller's sinogram, rows of U bins
+                    const size_t o = (size_t)v * P.U + ub;
+                    val.x = load_user(user, o, io.storage);   // (ub < U: U > Up - 4, and ub is a multiple of 4)
+                    if (ub + 1 < P.U) val.y = load_user(user, o + 1, io.storage);
+                    if (ub + 2 < P.U) val.z = load_user(user, o + 2, io.storage);
+                    if (ub + 3 < P.U) val.w = load_user(user, o + 3, io.storage);
+                } else {
+                    val = __ldg(reinterpret_cast<const float4 *>((s ? sino1 : sino0) + (size_t)v * Up + ub));
+                }
                 const float pl = vsh[buf][vv].P;   // the weights are in units of the view's plateau length
                 val.x = __fmul_rn(val.x, pl);
                 val.y = __fmul_rn(val.y, pl);
@@ -354,7 +364,14 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
                         if (solve && is_g[s]) P.glo[o] = (float)(v - (double)vh);
                     } else {
                         const float vh = __fadd_rn(vs.h, vs.l);   // the pair rounded to FP32
-                        outs[s][o] = vh;
+                        if (solve || !io.out) {
+                            outs[s][o] = vh;
+                        } else {   // the caller's image
+                            void *out = io.out + (size_t)pi * io.out_step;
+                            const size_t oc = (size_t)i * P.nx + j;
+                            if (io.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(out)[oc] = __float2bfloat16_rn(vh);
+                            else reinterpret_cast<float *>(out)[oc] = vh;
+                        }
                         if (solve && is_g[s]) P.glo[o] = __fsub_rn(vs.l, __fsub_rn(vh, vs.h));   // its error, exactly
                     }
                     if (want_se && s == 0) {   // pixel centre inside the ellipse (FP64, as the definition)
@@ -401,20 +418,20 @@ int backward_blocks(int nx, int ny, int dual, int parts)
 }
 
 template <bool DUAL, int FP>
-static int launch_bwd(const Launch &L, int mode, int bwin)
+static int launch_bwd(const Launch &L, int mode, int bwin, const Io &io = Io())
 {
     const int smem = 2 * (DUAL ? 2 : 1) * kBwdViewChunk * bwin * 4;
     int rc = func_attrs_once((const void *)k_backward<DUAL, FP>, 2 * (DUAL ? 2 : 1) * kBwdViewChunk * 256 * 4);
     if (rc) return rc;
-    k_backward<DUAL, FP><<<L.blocks, kBwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, mode);
+    k_backward<DUAL, FP><<<L.blocks, kBwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, mode, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }
 
-int launch_backward(const Launch &L, int mode, int bwin)
+int launch_backward(const Launch &L, int mode, int bwin, const Io &io)
 {
-    return L.bparts == kBwdViewParts ? launch_bwd<false, kBwdViewParts>(L, mode, bwin)
-                                     : launch_bwd<false, 0>(L, mode, bwin);
+    return L.bparts == kBwdViewParts ? launch_bwd<false, kBwdViewParts>(L, mode, bwin, io)
+                                     : launch_bwd<false, 0>(L, mode, bwin, io);
 }
 
 int launch_backward2(const Launch &L, int bwin)

@@ -10,19 +10,16 @@ constexpr int kVecPerThread = 4;
 constexpr int kVecPerBlock = kRedThreads * kVecPerThread;   // elements per block of the vector kernels
 
 // ------------------------------------------------------------ layout staging
-__device__ __forceinline__ float load_user(const void *p, size_t i, int storage)
-{
-    return storage == SUPCG_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p)[i])
-                                 : reinterpret_cast<const float *>(p)[i];
-}
-
 // Caller image [ny][nx] -> x [ny][nxp] and x^T [nx][nyp] (zero padding kept).
 __global__ void __launch_bounds__(256) k_stage_in(const Prob *__restrict__ probs, const int *__restrict__ prefix,
-                                                  int count, int which)
+                                                  int count, Io io)
 {
     __shared__ float sh[32][33];
     int local;
-    const Prob &P = probs[find_problem(prefix, count, blockIdx.x, &local)];
+    const int pi = find_problem(prefix, count, blockIdx.x, &local);
+    const Prob &P = probs[pi];
+    const void *in = io_in(io, P, pi);
+    const int storage = io_storage(io, P);
     const int tiles_j = (P.nx + 31) / 32;
     const int ti = local / tiles_j, tj = local - ti * tiles_j;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -30,14 +27,13 @@ __global__ void __launch_bounds__(256) k_stage_in(const Prob *__restrict__ probs
         const int i = ti * 32 + r, j = tj * 32 + tx;
         float v = 0.0f;
         if (i < P.ny && j < P.nx) {
-            v = load_user(P.in_user, (size_t)i * P.nx + j, P.storage);
-            (which ? P.g : P.x)[(size_t)i * P.nxp + j] = v;
-            if (!which && P.xlo) P.xlo[(size_t)i * P.nxp + j] = 0.0f;   // x_0 is exactly its FP32 value
-            if (!which && P.xm) P.xm[(size_t)i * P.nxp + (P.nx - 1 - j)] = v;
+            v = load_user(in, (size_t)i * P.nx + j, storage);
+            P.x[(size_t)i * P.nxp + j] = v;
+            if (P.xlo) P.xlo[(size_t)i * P.nxp + j] = 0.0f;   // x_0 is exactly its FP32 value
+            if (P.xm) P.xm[(size_t)i * P.nxp + (P.nx - 1 - j)] = v;
         }
         sh[r][tx] = v;
     }
-    if (which) return;
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
         const int j = tj * 32 + r, i = ti * 32 + tx;
@@ -48,32 +44,58 @@ __global__ void __launch_bounds__(256) k_stage_in(const Prob *__restrict__ probs
     }
 }
 
-int launch_stage_in(const Launch &L, int which)
+int launch_stage_in(const Launch &L, const Io &io)
 {
-    k_stage_in<<<L.blocks, 256, 0, L.st>>>(L.probs, L.prefix, L.count, which);
+    k_stage_in<<<L.blocks, 256, 0, L.st>>>(L.probs, L.prefix, L.count, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }
 
-// Caller sinogram [V][U] -> r (which 0) or bpad (which 1), pitch Up, zero padded.
-__global__ void __launch_bounds__(256) k_stage_sino(const Prob *__restrict__ probs, const int *__restrict__ prefix,
-                                                    int count, int which)
+// The start of a solve: every problem's scalars s0, its tickets and barriers at 0, and p = h = 0 (one launch
+// where each problem had five copies and fills).
+__global__ void __launch_bounds__(kRedThreads) k_init(const Prob *__restrict__ probs, const int *__restrict__ prefix,
+                                                      int count, Scal s0)
 {
     int local;
     const Prob &P = probs[find_problem(prefix, count, blockIdx.x, &local)];
-    float *dst = which ? P.bpad : P.r;
+    if (local == 0) {
+        if (threadIdx.x == 0) *P.sc = s0;
+        if (threadIdx.x < 16) P.counter[threadIdx.x] = 0;
+        if (threadIdx.x < 8) P.bar[threadIdx.x] = 0;
+    }
+    const size_t tot = (size_t)P.ny * P.nxp;   // a multiple of 4
+    const size_t e4 = (size_t)local * kRedThreads + threadIdx.x;
+    if (4 * e4 < tot) {
+        const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        reinterpret_cast<float4 *>(P.p)[e4] = zero;
+        reinterpret_cast<float4 *>(P.h)[e4] = zero;
+    }
+}
+
+int launch_init(const Launch &L, const Scal &s0)
+{
+    k_init<<<L.blocks, kRedThreads, 0, L.st>>>(L.probs, L.prefix, L.count, s0);
+    SUPCG_CUDA_TRY(cudaGetLastError());
+    return SUPCG_OK;
+}
+
+// Caller sinogram in_user2 [V][U] (FP32) -> bpad, pitch Up, zero padded.
+__global__ void __launch_bounds__(256) k_stage_sino(const Prob *__restrict__ probs, const int *__restrict__ prefix,
+                                                    int count)
+{
+    int local;
+    const Prob &P = probs[find_problem(prefix, count, blockIdx.x, &local)];
     const size_t tot = (size_t)P.V * P.Up;
     for (size_t e = (size_t)local * kVecPerBlock + threadIdx.x; e < tot && e < (size_t)(local + 1) * kVecPerBlock;
          e += kRedThreads) {
         const int v = (int)(e / P.Up), u = (int)(e - (size_t)v * P.Up);
-        const void *src = which ? P.in_user2 : P.in_user;
-        dst[e] = (u < P.U) ? load_user(src, (size_t)v * P.U + u, which ? SUPCG_F32 : P.storage) : 0.0f;
+        P.bpad[e] = (u < P.U) ? reinterpret_cast<const float *>(P.in_user2)[(size_t)v * P.U + u] : 0.0f;
     }
 }
 
-int launch_stage_sino(const Launch &L, int which)
+int launch_stage_sino(const Launch &L)
 {
-    k_stage_sino<<<L.blocks, kRedThreads, 0, L.st>>>(L.probs, L.prefix, L.count, which);
+    k_stage_sino<<<L.blocks, kRedThreads, 0, L.st>>>(L.probs, L.prefix, L.count);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }
@@ -122,27 +144,30 @@ int launch_rupdate(const Launch &L)
     return SUPCG_OK;
 }
 
-// Padded image (which 0: x, 1: g, 2: z, 3: tbar) -> caller image [ny][nx].
+// Padded image (which 0: x, 1: tbar, 2: g) -> caller image [ny][nx].
 __global__ void __launch_bounds__(256) k_store_out(const Prob *__restrict__ probs, const int *__restrict__ prefix,
-                                                   int count, int which)
+                                                   int count, int which, Io io)
 {
     int local;
-    const Prob &P = probs[find_problem(prefix, count, blockIdx.x, &local)];
-    const float *src = which == 0 ? P.x : (which == 1 ? P.g : (which == 2 ? P.z : P.tbar));
+    const int pi = find_problem(prefix, count, blockIdx.x, &local);
+    const Prob &P = probs[pi];
+    const float *src = which == 0 ? P.x : (which == 1 ? P.tbar : P.g);
+    void *out = io_out(io, P, pi);
+    const int storage = io_storage(io, P);
     const size_t tot = (size_t)P.ny * P.nxp;
     for (size_t e = (size_t)local * kVecPerBlock + threadIdx.x; e < tot && e < (size_t)(local + 1) * kVecPerBlock;
          e += kRedThreads) {
         const int i = (int)(e / P.nxp), j = (int)(e - (size_t)i * P.nxp);
         if (j >= P.nx) continue;
         const size_t o = (size_t)i * P.nx + j;
-        if (P.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(P.out_user)[o] = __float2bfloat16_rn(src[e]);
-        else reinterpret_cast<float *>(P.out_user)[o] = src[e];
+        if (storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(out)[o] = __float2bfloat16_rn(src[e]);
+        else reinterpret_cast<float *>(out)[o] = src[e];
     }
 }
 
-int launch_store_out(const Launch &L, int which)
+int launch_store_out(const Launch &L, int which, const Io &io)
 {
-    k_store_out<<<L.blocks, kRedThreads, 0, L.st>>>(L.probs, L.prefix, L.count, which);
+    k_store_out<<<L.blocks, kRedThreads, 0, L.st>>>(L.probs, L.prefix, L.count, which, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }

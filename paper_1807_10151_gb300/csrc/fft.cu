@@ -206,12 +206,17 @@ __device__ __forceinline__ float4 *fft_smem_df(float4 *a, float4 *b, int nvec, c
 //                 beyond nx/2 (the filtered rows are real);  z[2i] + i z[2i+1] =
 //                 IFFT(c) (the 1 / (nx ny) is folded into D).
 __global__ void __launch_bounds__(256) k_fft_rows(const Prob *__restrict__ probs, const int *__restrict__ prefix,
-                                                  int count, int inverse, int standalone)
+                                                  int count, int inverse, int standalone, Io io)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int local;
-    const Prob &P = probs[find_problem(prefix, count, blockIdx.x, &local)];
+    const int pi = find_problem(prefix, count, blockIdx.x, &local);
+    const Prob &P = probs[pi];
     if (!standalone && P.sc->done) return;
+    // standalone: g and z are the caller's FP32 images, rows of nx
+    const float *gsrc = standalone ? reinterpret_cast<const float *>(io.in + (size_t)pi * io.in_step) : P.g;
+    float *zdst = standalone ? reinterpret_cast<float *>(io.out + (size_t)pi * io.out_step) : P.z;
+    const int pitch = standalone ? P.nx : P.nxp;
     const int nx = P.nx, ny = P.ny, rpb = P.fft_rpb, hx = nx / 2 + 1;
     const int npairs = (ny + 1) / 2;
     float4 *a = reinterpret_cast<float4 *>(smem_raw);
@@ -226,9 +231,9 @@ __global__ void __launch_bounds__(256) k_fft_rows(const Prob *__restrict__ probs
         if (!inverse) {
             // inside a solve the gradient is the double-float pair (g, glo)
             const float *glo = standalone ? nullptr : P.glo;
-            const size_t ia = (size_t)ra * P.nxp + q, ib = (size_t)rb * P.nxp + q;
-            const float va = P.g[ia];
-            const float vb = rb < ny ? P.g[ib] : 0.0f;
+            const size_t ia = (size_t)ra * pitch + q, ib = (size_t)rb * pitch + q;
+            const float va = gsrc[ia];
+            const float vb = rb < ny ? gsrc[ib] : 0.0f;
             const float la = glo ? glo[ia] : 0.0f;
             const float lb = (glo && rb < ny) ? glo[ib] : 0.0f;
             a[e] = make_float4(va, la, vb, lb);
@@ -278,14 +283,14 @@ __global__ void __launch_bounds__(256) k_fft_rows(const Prob *__restrict__ probs
         auto put_z = [&](int e, float ha, float hb) {
             const int pr = e / nx, q = e - pr * nx;
             const int ra = 2 * (p0 + pr), rb = ra + 1;
-            const size_t ia = (size_t)ra * P.nxp + q, ib = (size_t)rb * P.nxp + q;
+            const size_t ia = (size_t)ra * pitch + q, ib = (size_t)rb * pitch + q;
             const float4 v = res[e];
             const float za = __fadd_rn(v.x, v.y);   // the pair rounded to FP32
-            P.z[ia] = za;
+            zdst[ia] = za;
             if (!standalone) df_acc_prod(s, za, ha);
             if (rb < ny) {
                 const float zb = __fadd_rn(v.z, v.w);
-                P.z[ib] = zb;
+                zdst[ib] = zb;
                 if (!standalone) df_acc_prod(s, zb, hb);
             }
         };
@@ -303,7 +308,6 @@ __global__ void __launch_bounds__(256) k_fft_rows(const Prob *__restrict__ probs
         if (!standalone) {
             __shared__ __align__(16) double red[40];
             __shared__ int flag;
-            const int pi = find_problem(prefix, count, blockIdx.x, &local);
             const double bs = block_sum_df<256>(s, red);
             if (threadIdx.x == 0) P.partial[local] = bs;
             const int nblk = prefix[pi + 1] - prefix[pi];
@@ -441,11 +445,11 @@ int launch_fft_dtab(const Launch &L)
     return SUPCG_OK;
 }
 
-int launch_fft_rows(const Launch &L, int inverse, int standalone, int smem)
+int launch_fft_rows(const Launch &L, int inverse, int standalone, int smem, const Io &io)
 {
     int rc = func_attrs_once((const void *)k_fft_rows, 200 * 1024);
     if (rc) return rc;
-    k_fft_rows<<<L.blocks, 256, smem, L.st>>>(L.probs, L.prefix, L.count, inverse, standalone);
+    k_fft_rows<<<L.blocks, 256, smem, L.st>>>(L.probs, L.prefix, L.count, inverse, standalone, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }

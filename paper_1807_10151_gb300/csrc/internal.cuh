@@ -231,7 +231,7 @@ struct Prob {
     double se_ax, se_ay;   // semi-axes of the SE ellipse, in pixels (horizontal, vertical)
     double gray_scale;     // ds / (V nx ny d^2): sum of b times this is the gray-level estimate
     int precond;           // 1: M of Eq. (3.2); 0: M = I
-    int storage;           // SUPCG_F32 / SUPCG_BF16 element type of in_user / out_user
+    int storage;           // SUPCG_F32 / SUPCG_BF16 element type of in_user / out_user (a solve: FP32)
     int stv_blocks;        // cooperative S_TV: blocks owned by this problem
     int fft_rpb, fft_cw;   // FFT rows per block / columns per block
     // solve buffers (images pitch nxp, transposed pitch nyp, sinograms pitch Up)
@@ -278,6 +278,30 @@ struct Prob {
     void *out_user;
     const void *in_user2;
 };
+
+// Caller-owned arrays of a standalone operator's batch, `step` bytes from one problem's to the next.  They are
+// kernel arguments, so that a call leaves the problems' descriptors on the device as they are; in == nullptr
+// (a solve): the problem's own in_user, out_user and storage.
+struct Io {
+    const char *in;
+    char *out;
+    size_t in_step, out_step;
+    int storage;
+};
+__device__ __forceinline__ const void *io_in(const Io &io, const Prob &P, int pi)
+{
+    return io.in ? io.in + (size_t)pi * io.in_step : P.in_user;
+}
+__device__ __forceinline__ void *io_out(const Io &io, const Prob &P, int pi)
+{
+    return io.in ? io.out + (size_t)pi * io.out_step : P.out_user;
+}
+__device__ __forceinline__ int io_storage(const Io &io, const Prob &P) { return io.in ? io.storage : P.storage; }
+__device__ __forceinline__ float load_user(const void *p, size_t i, int storage)
+{
+    return storage == SUPCG_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p)[i])
+                                 : reinterpret_cast<const float *>(p)[i];
+}
 
 // Map a block of a batched launch to (problem, block within problem).
 __device__ __forceinline__ int find_problem(const int *prefix, int count, int b, int *local)
@@ -704,8 +728,8 @@ struct Launch {
     cudaStream_t st;
 };
 
-int launch_forward(const Launch &L, const Launch &La, int which, int mode);   // La: every view's items
-int launch_backward(const Launch &L, int mode, int bwin);
+int launch_forward(const Launch &L, const Launch &La, int which, int mode, const Io &io = Io());   // La: every view's items
+int launch_backward(const Launch &L, int mode, int bwin, const Io &io = Io());   // BWD_PLAIN: caller sinogram -> caller image
 int launch_backward2(const Launch &L, int bwin);   // g from r and h from q in one pass
 int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side the longer one of the image
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st);
@@ -713,10 +737,11 @@ int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, i
 int backward_blocks(int nx, int ny, int dual, int parts);
 int encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims,
                  const cuuint64_t *strides_bytes, const cuuint32_t *box);
-int launch_stage_in(const Launch &L, int which);           // caller image -> x and x^T (0) or g (1)
-int launch_stage_sino(const Launch &L, int which);         // caller sinogram -> r (0, in_user) or bpad (1, in_user2)
-int launch_store_out(const Launch &L, int which);          // padded image (0 x, 1 g, 2 z, 3 tbar) -> caller
-int launch_fft_rows(const Launch &L, int inverse, int standalone, int smem);
+int launch_init(const Launch &L, const Scal &s0);           // every problem's scalars, counters and barriers; p = h = 0
+int launch_stage_in(const Launch &L, const Io &io = Io());  // caller image -> x and x^T
+int launch_stage_sino(const Launch &L);                     // caller sinogram in_user2 -> bpad
+int launch_store_out(const Launch &L, int which, const Io &io = Io());   // padded image (0 x, 1 tbar, 2 g) -> caller
+int launch_fft_rows(const Launch &L, int inverse, int standalone, int smem, const Io &io = Io());
 int launch_fft_cols(const Launch &L, int standalone, int smem);
 int launch_fft_wc(const Launch &L);                         // fills wc (once per workspace)
 int launch_fft_dtab(const Launch &L);                       // fills Dtab from mu, rho (once per solve or call)

@@ -365,7 +365,7 @@ constexpr int kFwdThreads = 64;   // two warps of 64 rays: 128 bins per block at
 template <bool MIRK>
 __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Prob *__restrict__ probs,
                                                                         const int *__restrict__ prefix, int count,
-                                                                        int which, int mode)
+                                                                        int which, int mode, Io io)
 {
     // proj_dyn: [warp][kFwdBufs][box: the image, (MIRK) its mirror][kRowsPerChunk][BW]
     __shared__ __align__(8) uint64_t bars[kFwdBufs * (kFwdThreads / 32)];   // one per staged box
@@ -449,8 +449,9 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
     auto emit = [&](int view, double a, int u) {
         if (mode == FWD_PLAIN) {
             const size_t o = (size_t)view * P.U + u;
-            if (P.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(P.out_user)[o] = __double2bfloat16(a);
-            else reinterpret_cast<float *>(P.out_user)[o] = (float)a;
+            void *out = io.out + (size_t)pi * io.out_step;
+            if (io.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(out)[o] = __double2bfloat16(a);
+            else reinterpret_cast<float *>(out)[o] = (float)a;
         } else if (mode == FWD_NORM) {
             const size_t o = (size_t)view * P.Up + u;
             const float qq = (float)a;
@@ -533,7 +534,7 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
 }
 
 template <bool MIRK>
-static int launch_forward_t(const Launch &L, int which, int mode)
+static int launch_forward_t(const Launch &L, int which, int mode, const Io &io)
 {
     // every problem's BW <= 256, so the warps' box buffers never exceed this size; with mirror
     // pairs each chunk holds two boxes
@@ -542,14 +543,14 @@ static int launch_forward_t(const Launch &L, int which, int mode)
     const int smem = (kFwdThreads / 32) * per_warp * L.bw_max * 4;
     int rc = func_attrs_once((const void *)k_forward<MIRK>, (kFwdThreads / 32) * per_warp * 256 * 4);
     if (rc) return rc;
-    k_forward<MIRK><<<L.blocks, kFwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, which, mode);
+    k_forward<MIRK><<<L.blocks, kFwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, which, mode, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }
 
-int launch_forward(const Launch &L, const Launch &La, int which, int mode)
+int launch_forward(const Launch &L, const Launch &La, int which, int mode, const Io &io)
 {
-    return L.mirror ? launch_forward_t<true>(L, which, mode) : launch_forward_t<false>(La, which, mode);
+    return L.mirror ? launch_forward_t<true>(L, which, mode, io) : launch_forward_t<false>(La, which, mode, io);
 }
 
 } // namespace supcg
