@@ -145,14 +145,13 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
     float Y[PX];
 #pragma unroll
     for (int e = 0; e < PX; ++e) Y[e] = __fsub_rn(P.cy, __int2float_rn(i0 + ly + kBwdRowStep * e));
-    // per pixel: FP32 sum of up to four views (t2, pixels in pairs), folded into a Kahan-compensated
-    // pair (part, comp) that runs over all views; FP64 only for the final value (the FP64 pipe is narrow)
-    float part[NS * PX], comp[NS * PX];
-    uint64_t t2[NS * PX / 2];
+    // per pixel: FP32 sum of up to four views (t2), folded into a Kahan-compensated pair (part, comp)
+    // that runs over all views, FP64 only for the final value (the FP64 pipe is narrow).  The views are
+    // issue-bound, so all three are kept as pixel pairs and the fold takes half the instructions; it
+    // also ends the repacking that spilled 28 to 112 bytes (171.9 -> 168.3 us for eight 243^2 / 320)
+    uint64_t part2[NS * PX / 2], comp2[NS * PX / 2], t2[NS * PX / 2];
 #pragma unroll
-    for (int e = 0; e < NS * PX; ++e) part[e] = comp[e] = 0.0f;
-#pragma unroll
-    for (int h = 0; h < NS * PX / 2; ++h) t2[h] = pk2(0.0f, 0.0f);
+    for (int h = 0; h < NS * PX / 2; ++h) t2[h] = part2[h] = comp2[h] = pk2(0.0f, 0.0f);
     uint64_t Y2[PX / 2];
 #pragma unroll
     for (int h = 0; h < PX / 2; ++h) Y2[h] = pk2(Y[2 * h], Y[2 * h + 1]);
@@ -282,24 +281,25 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
                     }
                 }
             }
-            float t4[NS * PX];
 #pragma unroll
-            for (int h = 0; h < NS * PX / 2; ++h) {
-                upk2(t2[h], t4[2 * h], t4[2 * h + 1]);
+            for (int h = 0; h < NS * PX / 2; ++h) {   // the fold, two pixels per instruction
+                const uint64_t y = sub2_rn(t2[h], comp2[h]);
+                const uint64_t tt = add2_rn(part2[h], y);
+                comp2[h] = sub2_rn(sub2_rn(tt, part2[h]), y);
+                part2[h] = tt;
                 t2[h] = pk2(0.0f, 0.0f);
-            }
-#pragma unroll
-            for (int e = 0; e < NS * PX; ++e) {
-                const float y = __fsub_rn(t4[e], comp[e]);
-                const float tt = __fadd_rn(part[e], y);
-                comp[e] = __fsub_rn(__fsub_rn(tt, part[e]), y);
-                part[e] = tt;
             }
         }
         __syncthreads();
     }
     // the Kahan pair as a double-float value part - comp (|comp| <= ulp(part) / 2); the
     // groups' and the parts' sums are added in double-float arithmetic, in a fixed order
+    float part[NS * PX], comp[NS * PX];
+#pragma unroll
+    for (int h = 0; h < NS * PX / 2; ++h) {
+        upk2(part2[h], part[2 * h], part[2 * h + 1]);
+        upk2(comp2[h], comp[2 * h], comp[2 * h + 1]);
+    }
     if (bad) atomicExch(&bad_sh, 1);
     __syncthreads();
     if (grp == 1)
