@@ -82,7 +82,7 @@ static int fft_factor(int n, int *rad)
 
 // ------------------------------------------------------------------ objects
 constexpr int kInlineTrials = 64;   // S_TV trial counts read back together with the scalars
-enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWD2, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
+enum { KT_FWD, KT_FWDA, KT_BWD, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
 
 struct Workspace {
     int count = 0;
@@ -99,6 +99,7 @@ struct Workspace {
     int bwin = 0;
     int bw_max = 0;
     int bparts = 0;             // view parts of every problem's backprojector, 0 if they differ
+    int bwd_ti = kBwdTileI;     // rows of its tiles
     int mirror = 0;             // 1: some problem has mirror pairs of views
     int stv_ti = 0;             // rows of k_stv_tile's tiles; 0: the images do not fit, S_TV walks them in memory
     bool wc_ready = false;      // the problems' frequency tables are filled
@@ -123,6 +124,7 @@ struct Workspace {
         l.blocks = blocks[kt];
         l.bw_max = bw_max;
         l.bparts = bparts;
+        l.bwd_ti = bwd_ti;
         l.mirror = mirror;
         l.st = st;
         return l;
@@ -589,14 +591,19 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
 
     // blocks per problem for every kernel type
     std::vector<std::vector<int>> nb(KT_COUNT, std::vector<int>(w->count));
-    long long stv_want = 0;
+    long long stv_want = 0, bwd32 = 0;
+    w->bparts = gs[0]->bparts;
+    for (int c = 0; c < w->count; ++c) {
+        bwd32 += backward_blocks(gs[c]->nx, gs[c]->ny, gs[c]->bparts, kBwdTileI);
+        if (gs[c]->bparts != w->bparts) w->bparts = 0;
+    }
+    w->bwd_ti = w->bparts == kBwdViewParts ? bwd_tile_rows(bwd32, nsm) : kBwdTileI;
     std::vector<long long> npx(w->count);
     for (int c = 0; c < w->count; ++c) {
         const supcg_geometry g = gs[c];
         nb[KT_FWD][c] = (g->nfw + 1) / 2;
         nb[KT_FWDA][c] = (g->nfw_all + 1) / 2;
-        nb[KT_BWD][c] = backward_blocks(g->nx, g->ny, 0, g->bparts);
-        nb[KT_BWD2][c] = backward_blocks(g->nx, g->ny, 1, g->bparts);
+        nb[KT_BWD][c] = backward_blocks(g->nx, g->ny, g->bparts, w->bwd_ti);
         nb[KT_VEC][c] = (int)(((long long)g->ny * g->nxp + 1023) / 1024);
         nb[KT_TR][c] = ((g->ny + 31) / 32) * ((g->nx + 31) / 32);
         // FFT: enough blocks to fill the device, each a few row pairs / stored columns
@@ -685,7 +692,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
                                 sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, 0,
                                 npart * 8, 16 * 4, 8 * 4, (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 8,
                                 2 * (size_t)g->bparts * img * 8,
-                                (size_t)std::max(nb[KT_BWD][c], nb[KT_BWD2][c]) * 4, img * 4, img * 4,
+                                (size_t)nb[KT_BWD][c] * 4, img * 4, img * 4,
                                 mir * img * 4, mir * imgT * 4, mir * img * 4, mir * imgT * 4,
                                 img * 4, imgT * 4, mir * img * 4, mir * imgT * 4, sino * 8, sino * 8,
                                 (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 16};
@@ -706,7 +713,6 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.counter = (unsigned *)ptrs[14]; P.bar = (unsigned *)ptrs[15]; P.Dtab = (float2 *)ptrs[16];
         P.bsplit = (float2 *)ptrs[17]; P.tilecnt = (unsigned *)ptrs[18]; P.xlo = (float *)ptrs[19];
         P.bparts = g->bparts;
-        w->bparts = (c == 0 || w->bparts == g->bparts) ? g->bparts : 0;
         P.glo = (float *)ptrs[20];
         P.xm = mir ? (float *)ptrs[21] : nullptr;
         P.xmT = mir ? (float *)ptrs[22] : nullptr;
@@ -1171,7 +1177,7 @@ static int enqueue_body(Workspace *w, const supcg_params *p, cudaStream_t st, in
     }
     // g = R^T r, and h = R^T q of the previous step (A p for this step's beta; the previous alpha
     // took p^T A p from ||q||^2), one pass over the views for both
-    LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward2(w->L(KT_BWD2, st), w->bwin));
+    LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward2(w->L(KT_BWD, st), w->bwin));
     if (p->precondition) {                                                      // z = M g; its last pass
         if ((rc = enqueue_precond_k(w, st))) return rc;                         // also forms beta
     } else {

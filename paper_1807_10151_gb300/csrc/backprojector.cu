@@ -2,7 +2,7 @@
 // equations R^T R x = R^T b).
 //
 // Backward (pixel-driven, gather over bins, no atomics).  A tile of 32 x 32
-// pixels is shared by P.bparts blocks (the geometry's view parts, 1 .. 8),
+// pixels (16 or 8 rows in small grids) is shared by P.bparts blocks (the geometry's view parts, 1 .. 8),
 // each taking a contiguous part of the view chunks; for chunks of 32 views the bins that the tile projects
 // onto are staged in shared memory with 16-byte vector loads; every pixel
 // gathers the two (three) bins nearest to its projected centre with the same
@@ -22,15 +22,17 @@ constexpr int kBwdGroup = 128;                                           // thre
 constexpr int kBwdThreads = kBwdSplit * kBwdGroup;
 constexpr int kBwdRowStep = kBwdGroup / kBwdTileJ;                       // 4
 
-// Tiles of 32 x 32 pixels, 8 per thread, over one sinogram or, DUAL, two (the
+// Tiles of TI x 32 pixels, TI / 4 per thread, over one sinogram or, DUAL, two (the
 // solver's R^T r and R^T q in one pass: each pixel's weights evaluated once and
 // applied to both; twice the sums per thread, so two blocks per SM instead of
-// three).  Either way a pixel sums its views in the same order (same groups,
-// folds and parts), so each output has the same bits as from the one-sinogram kernel.
-template <bool DUAL>
+// three).  Either way, and for every TI, a pixel sums its views in the same order (same
+// groups, folds and parts), so each output has the same bits.  TI = 32 spreads a view's
+// constants and staging over the most pixels; images whose 32-row tiles would leave SMs
+// without a block take 16 or 8 rows (bwd_tile_rows).
+template <bool DUAL, int TILE>
 struct BwdShape {
     static constexpr int NS = DUAL ? 2 : 1;                        // sinograms
-    static constexpr int TI = kBwdTileI;                           // tile rows
+    static constexpr int TI = TILE;                                // tile rows
     static constexpr int PX = TI * kBwdTileJ / kBwdGroup;          // pixels per thread
 };
 
@@ -108,12 +110,12 @@ __device__ __forceinline__ void bwd_view_x2(const ViewP &vp, float pb0, const ui
 // deferred to this pass: alpha takes p^T A p from the forward projector's ||q||^2).
 // FIXED_PARTS: the view parts per tile when every problem of the launch has that
 // (default) number, so the part arithmetic is compile-time; 0: each problem's own.
-template <bool DUAL, int FIXED_PARTS>
+template <bool DUAL, int FIXED_PARTS, int TILE>
 __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Prob *__restrict__ probs,
                                                           const int *__restrict__ prefix, int count, int mode,
                                                           Io io)
 {
-    constexpr int NS = BwdShape<DUAL>::NS, TI = BwdShape<DUAL>::TI, PX = BwdShape<DUAL>::PX;
+    constexpr int NS = BwdShape<DUAL, TILE>::NS, TI = BwdShape<DUAL, TILE>::TI, PX = BwdShape<DUAL, TILE>::PX;
     // proj_dyn: [2][NS][kBwdViewChunk][bwin] sinogram windows
     __shared__ ViewP vsh[2][kBwdViewChunk];
     __shared__ int ulo_sh[2][kBwdViewChunk];
@@ -410,34 +412,45 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
     }
 }
 
-// Blocks per problem: `parts` per pixel tile.
-int backward_blocks(int nx, int ny, int dual, int parts)
+// Blocks per problem: `parts` per pixel tile of `ti` rows.
+int backward_blocks(int nx, int ny, int parts, int ti)
 {
-    const int ti = dual ? BwdShape<true>::TI : BwdShape<false>::TI;
     return parts * ((ny + ti - 1) / ti) * ((nx + kBwdTileJ - 1) / kBwdTileJ);
 }
 
-template <bool DUAL, int FP>
-static int launch_bwd(const Launch &L, int mode, int bwin, const Io &io = Io())
+// Rows of a launch's tiles, from its number of blocks with 32 rows: the lowest with which the grid still is
+// no more than two blocks per SM, which all run at once (two of the solver's dual pass fit).  A block's time
+// is a serial chain of view groups whose length hardly falls below its rows' share while the SM has nothing
+// else to issue.  One R^T y with 32 rows and as chosen, us: 64^2 / 90 views 16.4 and 9.6 (8 rows),
+// 128^2 / 180 20.6 and 14.4 (8), 160^2 / 200 20.6 and 16.4 (16), 192^2 / 240 20.6 and 18.5 (16); from
+// 224^2 / 300 on (28.7) the 32-row grid has more than one block per SM and stays.  The solver's dual pass at 64^2:
+// 25.6 and 14.6.
+int bwd_tile_rows(long long blocks32, int nsm)
+{
+    return 4 * blocks32 <= 2 * nsm ? 8 : (2 * blocks32 <= 2 * nsm ? 16 : kBwdTileI);
+}
+
+template <bool DUAL, int FP, int TILE>
+static int launch_bwd(const Launch &L, int mode, int bwin, const Io &io)
 {
     const int smem = 2 * (DUAL ? 2 : 1) * kBwdViewChunk * bwin * 4;
-    int rc = func_attrs_once((const void *)k_backward<DUAL, FP>, 2 * (DUAL ? 2 : 1) * kBwdViewChunk * 256 * 4);
+    int rc = func_attrs_once((const void *)k_backward<DUAL, FP, TILE>, 2 * (DUAL ? 2 : 1) * kBwdViewChunk * 256 * 4);
     if (rc) return rc;
-    k_backward<DUAL, FP><<<L.blocks, kBwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, mode, io);
+    k_backward<DUAL, FP, TILE><<<L.blocks, kBwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, mode, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }
 
-int launch_backward(const Launch &L, int mode, int bwin, const Io &io)
+template <bool DUAL>
+static int launch_bwd_any(const Launch &L, int mode, int bwin, const Io &io)
 {
-    return L.bparts == kBwdViewParts ? launch_bwd<false, kBwdViewParts>(L, mode, bwin, io)
-                                     : launch_bwd<false, 0>(L, mode, bwin, io);
+    if (L.bparts != kBwdViewParts) return launch_bwd<DUAL, 0, kBwdTileI>(L, mode, bwin, io);
+    if (L.bwd_ti == 8) return launch_bwd<DUAL, kBwdViewParts, 8>(L, mode, bwin, io);
+    if (L.bwd_ti == 16) return launch_bwd<DUAL, kBwdViewParts, 16>(L, mode, bwin, io);
+    return launch_bwd<DUAL, kBwdViewParts, kBwdTileI>(L, mode, bwin, io);
 }
 
-int launch_backward2(const Launch &L, int bwin)
-{
-    return L.bparts == kBwdViewParts ? launch_bwd<true, kBwdViewParts>(L, BWD_G, bwin)
-                                     : launch_bwd<true, 0>(L, BWD_G, bwin);
-}
+int launch_backward(const Launch &L, int mode, int bwin, const Io &io) { return launch_bwd_any<false>(L, mode, bwin, io); }
+int launch_backward2(const Launch &L, int bwin) { return launch_bwd_any<true>(L, BWD_G, bwin, Io()); }
 
 } // namespace supcg

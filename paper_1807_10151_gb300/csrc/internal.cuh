@@ -724,6 +724,7 @@ struct Launch {
     int blocks;            // total blocks
     int bw_max;            // widest forward box (floats) among the problems
     int bparts;            // backprojector view parts shared by every problem, 0 if they differ
+    int bwd_ti;            // backprojector tile rows (with the default view parts)
     int mirror;            // 1: some problem has mirror pairs of views (the forward projector's paired variant)
     cudaStream_t st;
 };
@@ -734,7 +735,8 @@ int launch_backward2(const Launch &L, int bwin);   // g from r and h from q in o
 int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side the longer one of the image
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st);
 int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
-int backward_blocks(int nx, int ny, int dual, int parts);
+int backward_blocks(int nx, int ny, int parts, int ti);
+int bwd_tile_rows(long long blocks32, int nsm);   // tile rows of a launch that has blocks32 blocks with 32 rows
 int encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims,
                  const cuuint64_t *strides_bytes, const cuuint32_t *box);
 int launch_init(const Launch &L, const Scal &s0);           // every problem's scalars, counters and barriers; p = h = 0
