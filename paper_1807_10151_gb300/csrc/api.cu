@@ -82,7 +82,7 @@ static int fft_factor(int n, int *rad)
 
 // ------------------------------------------------------------------ objects
 constexpr int kInlineTrials = 64;   // S_TV trial counts read back together with the scalars
-enum { KT_FWD, KT_FWDA, KT_BWD, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
+enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWDP, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SINO, KT_STV, KT_STVT, KT_TV, KT_COUNT };
 
 struct Workspace {
     int count = 0;
@@ -100,6 +100,8 @@ struct Workspace {
     int bw_max = 0;
     int bparts = 0;             // view parts of every problem's backprojector, 0 if they differ
     int bwd_ti = kBwdTileI;     // rows of its tiles
+    int bwdp_ti = kPairTileI;   // the same over mirror pairs
+    int bwp = 0;                // widest window there
     int mirror = 0;             // 1: some problem has mirror pairs of views
     int stv_ti = 0;             // rows of k_stv_tile's tiles; 0: the images do not fit, S_TV walks them in memory
     bool wc_ready = false;      // the problems' frequency tables are filled
@@ -125,6 +127,7 @@ struct Workspace {
         l.bw_max = bw_max;
         l.bparts = bparts;
         l.bwd_ti = bwd_ti;
+        l.bwdp_ti = bwdp_ti;
         l.mirror = mirror;
         l.st = st;
         return l;
@@ -164,6 +167,8 @@ struct supcg_geometry_s {
     // gives pixel (i, j), so the forward projector evaluates the weights once for both.
     // mirror[v] = w for the pair's first view (cos > 0), -2 for its second, -1 unpaired.
     std::vector<int> mirror;
+    int2 *dbitems = nullptr;        // backprojector items (see backproject_pairs.cu), or none
+    int nbi = 0, bwp = 0;           // their number, and the bins that a window of theirs holds
     int *dmirror = nullptr;         // device copy: the partner of a pair's first view, else -1
     int npairs = 0;
     int *dborder = nullptr;         // forward warp items in launch order, at most V x ceil(U / 32)
@@ -380,7 +385,7 @@ extern "C" int supcg_create_geometry(int nx, int ny, double pixel_size, int n_vi
     split(uc, Q, &g->uc_hi, &g->uc_lo);
     g->views.resize(n_views);
     std::vector<int> A, B;
-    double maxE = 0.0, span_bwd = 0.0, max_small = fabs((double)g->uc_lo);
+    double maxE = 0.0, span_bwd = 0.0, span_pair = 0.0, max_small = fabs((double)g->uc_lo);
     double mcl = 0.0, msl = 0.0;
     for (int v = 0; v < n_views; ++v) {
         const double c = vcos[v], s = vsin[v];
@@ -422,6 +427,7 @@ extern "C" int supcg_create_geometry(int nx, int ny, double pixel_size, int n_vi
         g->views[v] = vp;
         maxE = std::max(maxE, (double)vp.E);
         span_bwd = std::max(span_bwd, (kBwdTileJ - 1) * fabs((double)vp.cu) + (kBwdTileI - 1) * fabs((double)vp.su));
+        span_pair = std::max(span_pair, (kBwdTileJ - 1) * fabs((double)vp.cu) + (kPairTileI - 1) * fabs((double)vp.su));
     }
     max_small += mcl * (cx + 1.0) + msl * (cy + 1.0);
     // the three bins nearest a pixel's centre must cover its footprint, and a
@@ -490,6 +496,27 @@ extern "C" int supcg_create_geometry(int nx, int ny, double pixel_size, int n_vi
     if ((rc = upload_block_order(g))) {
         supcg_destroy_geometry(g);
         return rc;
+    }
+    // R^T y over mirror pairs where three quarters of the views have one (an unpaired view costs as much as a
+    // pair there) and two blocks' windows fit an SM.  At that share, us: one R^T y at 512^2 / 720 views 141
+    // against the general kernel's 166, at 256^2 / 360 34.4 and 34.9, the solver's pass 193 and 220, 44 and 49;
+    // with all views but two paired 119, 28.7, 161 and 38 (general: the same as above).
+    g->bwp = round_up((int)ceil(span_pair + 11.0), 4);
+    if (8LL * g->npairs >= 3LL * n_views && g->bwp <= kPairWindowMax) {
+        std::vector<int2> items;
+        for (int v = 0; v < n_views; ++v)
+            if (g->mirror[v] >= 0) items.push_back(make_int2(v, g->mirror[v]));
+        for (int v = 0; v < n_views; ++v)
+            if (g->mirror[v] == -1) items.push_back(make_int2(v, -1));
+        if (cudaMalloc(&g->dbitems, sizeof(int2) * items.size()) != cudaSuccess) {
+            supcg_destroy_geometry(g);
+            return SUPCG_ERR_NOMEM;
+        }
+        if (cudaMemcpy(g->dbitems, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+            supcg_destroy_geometry(g);
+            return SUPCG_ERR_CUDA;
+        }
+        g->nbi = (int)items.size();
     }
     *out = g;
     return SUPCG_OK;
@@ -560,6 +587,7 @@ extern "C" int supcg_destroy_geometry(supcg_geometry g)
     if (g->dviews) cudaFree(g->dviews);
     if (g->dvlist) cudaFree(g->dvlist);
     if (g->dmirror) cudaFree(g->dmirror);
+    if (g->dbitems) cudaFree(g->dbitems);
     if (g->dborder) cudaFree(g->dborder);
     if (g->dborder_all) cudaFree(g->dborder_all);
     if (g->host_db) cudaFree(g->host_db);
@@ -594,16 +622,19 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
     long long stv_want = 0, bwd32 = 0;
     w->bparts = gs[0]->bparts;
     for (int c = 0; c < w->count; ++c) {
-        bwd32 += backward_blocks(gs[c]->nx, gs[c]->ny, gs[c]->bparts, kBwdTileI);
+        bwd32 += gs[c]->nbi ? backward_pairs_blocks(gs[c]->nx, gs[c]->ny, gs[c]->bparts, kPairTileI)
+                            : backward_blocks(gs[c]->nx, gs[c]->ny, gs[c]->bparts, kBwdTileI);
         if (gs[c]->bparts != w->bparts) w->bparts = 0;
     }
     w->bwd_ti = w->bparts == kBwdViewParts ? bwd_tile_rows(bwd32, nsm) : kBwdTileI;
+    w->bwdp_ti = w->bwd_ti / 2;   // (16 rows on both sides are the pixels of 32)
     std::vector<long long> npx(w->count);
     for (int c = 0; c < w->count; ++c) {
         const supcg_geometry g = gs[c];
         nb[KT_FWD][c] = (g->nfw + 1) / 2;
         nb[KT_FWDA][c] = (g->nfw_all + 1) / 2;
-        nb[KT_BWD][c] = backward_blocks(g->nx, g->ny, g->bparts, w->bwd_ti);
+        nb[KT_BWD][c] = g->nbi ? 0 : backward_blocks(g->nx, g->ny, g->bparts, w->bwd_ti);
+        nb[KT_BWDP][c] = g->nbi ? backward_pairs_blocks(g->nx, g->ny, g->bparts, w->bwdp_ti) : 0;
         nb[KT_VEC][c] = (int)(((long long)g->ny * g->nxp + 1023) / 1024);
         nb[KT_TR][c] = ((g->ny + 31) / 32) * ((g->nx + 31) / 32);
         // FFT: enough blocks to fill the device, each a few row pairs / stored columns
@@ -692,7 +723,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
                                 sino * 4, sino * 4, sino * 4, (size_t)g->ny * g->nx * 16, 0,
                                 npart * 8, 16 * 4, 8 * 4, (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 8,
                                 2 * (size_t)g->bparts * img * 8,
-                                (size_t)nb[KT_BWD][c] * 4, img * 4, img * 4,
+                                (size_t)std::max(nb[KT_BWD][c], nb[KT_BWDP][c]) * 4, img * 4, img * 4,
                                 mir * img * 4, mir * imgT * 4, mir * img * 4, mir * imgT * 4,
                                 img * 4, imgT * 4, mir * img * 4, mir * imgT * 4, sino * 8, sino * 8,
                                 (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 16};
@@ -736,6 +767,8 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.cx = g->cx; P.cy = g->cy; P.uc = g->uc; P.uc_hi = g->uc_hi; P.uc_lo = g->uc_lo;
         P.bwin = g->bwin;
         w->bwin = std::max(w->bwin, g->bwin);
+        P.bwp = g->bwp; P.nbi = g->nbi; P.bitems = g->dbitems;
+        if (g->nbi) w->bwp = std::max(w->bwp, g->bwp);
         w->bw_max = std::max(w->bw_max, g->BW);
         P.views = g->dviews; P.vlist = g->dvlist;
         P.fx = g->fx; P.fy = g->fy;
@@ -896,6 +929,16 @@ extern "C" int supcg_project(supcg_geometry g, const void *d_x, void *d_y, int b
     return launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_PLAIN, io);
 }
 
+// R^T y (dual: g from r and h from q in one pass): the problems with mirror pairs, then the others, each if any.
+static int enqueue_backward(Workspace *w, cudaStream_t st, bool dual, int mode, const Io &io)
+{
+    int rc = SUPCG_OK;
+    if (w->blocks[KT_BWDP]) rc = launch_backward_pairs(w->L(KT_BWDP, st), dual, mode, w->bwp, io);
+    if (!rc && w->blocks[KT_BWD])
+        rc = dual ? launch_backward2(w->L(KT_BWD, st), w->bwin) : launch_backward(w->L(KT_BWD, st), mode, w->bwin, io);
+    return rc;
+}
+
 extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, int batch, void *stream)
 {
     if (!g || !d_x || !d_y || batch < 1) return SUPCG_ERR_ARG;
@@ -909,10 +952,10 @@ extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, i
     if (scope.rc) return scope.rc;
     // straight into the caller's image, unless it overlaps the sinogram still being read
     const char *y = (const char *)d_y, *x = (const char *)d_x;
-    if (y + batch * m * es <= x || x + batch * n * es <= y) return launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin, io);
+    if (y + batch * m * es <= x || x + batch * n * es <= y) return enqueue_backward(w, st, false, BWD_PLAIN, io);
     Io to_g = io;
     to_g.out = nullptr;
-    if ((rc = launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin, to_g))) return rc;
+    if ((rc = enqueue_backward(w, st, false, BWD_PLAIN, to_g))) return rc;
     return launch_store_out(w->L(KT_VEC, st), 2, io);
 }
 
@@ -1177,7 +1220,7 @@ static int enqueue_body(Workspace *w, const supcg_params *p, cudaStream_t st, in
     }
     // g = R^T r, and h = R^T q of the previous step (A p for this step's beta; the previous alpha
     // took p^T A p from ||q||^2), one pass over the views for both
-    LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward2(w->L(KT_BWD, st), w->bwin));
+    LAUNCH(SUPCG_KIND_BACKWARD, st, enqueue_backward(w, st, true, BWD_G, Io()));
     if (p->precondition) {                                                      // z = M g; its last pass
         if ((rc = enqueue_precond_k(w, st))) return rc;                         // also forms beta
     } else {
@@ -1194,7 +1237,7 @@ static int enqueue_init(Workspace *w, const supcg_params *p, cudaStream_t st)
 {
     int rc;
     LAUNCH(SUPCG_KIND_FORWARD, st, launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_RESID));
-    LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward(w->L(KT_BWD, st), BWD_G, w->bwin));
+    LAUNCH(SUPCG_KIND_BACKWARD, st, enqueue_backward(w, st, false, BWD_G, Io()));
     if (p->precondition) {
         if ((rc = enqueue_precond_k(w, st))) return rc;
     } else {

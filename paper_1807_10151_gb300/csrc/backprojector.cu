@@ -1,5 +1,6 @@
 // The exact transpose R^T y of the forward projection (Eq. (2.2): normal
-// equations R^T R x = R^T b).
+// equations R^T R x = R^T b), for any set of views; sets of mirror pairs take
+// backproject_pairs.cu.
 //
 // Backward (pixel-driven, gather over bins, no atomics).  A tile of 32 x 32
 // pixels (16 or 8 rows in small grids) is shared by P.bparts blocks (the geometry's view parts, 1 .. 8),
@@ -8,7 +9,7 @@
 // gathers the two (three) bins nearest to its projected centre with the same
 // weight evaluated on the same FP32 operands as the forward kernel.  The last
 // block of a tile to finish adds the parts' double-float sums in part order.
-#include "internal.cuh"
+#include "backward.cuh"
 
 namespace supcg {
 
@@ -17,11 +18,6 @@ namespace supcg {
 extern __shared__ __align__(128) float proj_dyn[];
 
 // ============================================================ backward
-constexpr int kBwdSplit = 2;                                             // thread groups splitting the views
-constexpr int kBwdGroup = 128;                                           // threads per group
-constexpr int kBwdThreads = kBwdSplit * kBwdGroup;
-constexpr int kBwdRowStep = kBwdGroup / kBwdTileJ;                       // 4
-
 // Tiles of TI x 32 pixels, TI / 4 per thread, over one sinogram or, DUAL, two (the
 // solver's R^T r and R^T q in one pass: each pixel's weights evaluated once and
 // applied to both; twice the sums per thread, so two blocks per SM instead of
@@ -122,7 +118,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
     __shared__ int kind_sh[2][kBwdViewChunk];   // variant: three bins (1) / two bins (2), + 3 if a window check is needed; axis 3
     __shared__ float2 comb[kBwdGroup * NS * PX];   // second group's sums, combined by the first
     __shared__ __align__(16) double red[40];
-    __shared__ int bad_sh;
+    __shared__ int bad_sh, last_sh;
 
     int local;
     const int pi = find_problem(prefix, count, blockIdx.x, &local);
@@ -294,122 +290,18 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
         }
         __syncthreads();
     }
-    // the Kahan pair as a double-float value part - comp (|comp| <= ulp(part) / 2); the
-    // groups' and the parts' sums are added in double-float arithmetic, in a fixed order
     float part[NS * PX], comp[NS * PX];
 #pragma unroll
     for (int h = 0; h < NS * PX / 2; ++h) {
         upk2(part2[h], part[2 * h], part[2 * h + 1]);
         upk2(comp2[h], comp[2 * h], comp[2 * h + 1]);
     }
-    if (bad) atomicExch(&bad_sh, 1);
-    __syncthreads();
-    if (grp == 1)
-#pragma unroll
-        for (int e = 0; e < NS * PX; ++e) comb[e * kBwdGroup + tg] = make_float2(part[e], -comp[e]);
-    __syncthreads();
-    // this part's sums; the tile's last part to finish adds them in part order
-    const size_t img = (size_t)P.ny * P.nxp;
-    if (grp == 0)
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int e = 0; e < PX; ++e) {
-                const int i = i0 + ly + kBwdRowStep * e;
-                if (i < P.ny && j < P.nx) {
-                    const float2 o2 = comb[(s * PX + e) * kBwdGroup + tg];
-                    const df v = df_add(df{part[s * PX + e], -comp[s * PX + e]}, df{o2.x, o2.y});
-                    P.bsplit[(size_t)(s * parts + vpart) * img + (size_t)i * P.nxp + j] = make_float2(v.h, v.l);
-                }
-            }
-    if (t == 0 && bad_sh && P.sc) atomicExch(&P.sc->status, (int)SUPCG_ERR_UNSUPPORTED);
-    __shared__ int last_sh;
-    if (!last_block(&P.tilecnt[tile], parts, &last_sh)) return;
-    // output s: the gradient (g from r) or h from q
-    const bool is_g[2] = {DUAL || mode != BWD_H, false};
-    float *outs[2] = {(!DUAL && mode == BWD_H) ? P.h : P.g, P.h};
-    // Bayesian criterion (Eq. (2.3)): g = r^2 R^T r + (x - mu_X), h = r^2 R^T q + p, and
-    // ||x - mu_X||^2 for f.  With a reference image, the selective error of Eq. (4.1) of
-    // x = x_{k+1/2} over the centred ellipse S (this pass reads x anyway).
-    const bool solve = DUAL || mode != BWD_PLAIN;
-    const bool bayes = solve && P.r2 > 0.0;
-    const bool want_se = (DUAL || mode == BWD_G) && P.se_ref != nullptr && !P.sc->init;
-    const double muX = bayes ? P.sc->muX : 0.0;
-    double sx = 0.0, sse = 0.0;
-    if (grp == 0)
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int e = 0; e < PX; ++e) {
-                const int i = i0 + ly + kBwdRowStep * e;
-                if (i < P.ny && j < P.nx) {
-                    const size_t o = (size_t)i * P.nxp + j;
-                    float2 pv[kBwdMaxParts];   // the other blocks' sums: read past L1
-#pragma unroll
-                    for (int h = 0; h < kBwdMaxParts; ++h)
-                        if (h < parts) pv[h] = __ldcg(P.bsplit + (size_t)(s * parts + h) * img + o);
-                    df vs = {0.0f, 0.0f};
-#pragma unroll
-                    for (int h = 0; h < kBwdMaxParts; ++h)
-                        if (h < parts) vs = df_add(vs, df{pv[h].x, pv[h].y});
-                    if (bayes) {
-                        double v = (double)vs.h + (double)vs.l;
-                        if (is_g[s]) {
-                            const double dx = (double)P.x[o] - muX;
-                            v = P.r2 * v + dx;
-                            sx += dx * dx;
-                        } else {
-                            v = P.r2 * v + (double)P.p[o];
-                        }
-                        const float vh = (float)v;
-                        outs[s][o] = vh;
-                        if (solve && is_g[s]) P.glo[o] = (float)(v - (double)vh);
-                    } else {
-                        const float vh = __fadd_rn(vs.h, vs.l);   // the pair rounded to FP32
-                        if (solve || !io.out) {
-                            outs[s][o] = vh;
-                        } else {   // the caller's image
-                            void *out = io.out + (size_t)pi * io.out_step;
-                            const size_t oc = (size_t)i * P.nx + j;
-                            if (io.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(out)[oc] = __float2bfloat16_rn(vh);
-                            else reinterpret_cast<float *>(out)[oc] = vh;
-                        }
-                        if (solve && is_g[s]) P.glo[o] = __fsub_rn(vs.l, __fsub_rn(vh, vs.h));   // its error, exactly
-                    }
-                    if (want_se && s == 0) {   // pixel centre inside the ellipse (FP64, as the definition)
-                        const double ex = ((double)j - 0.5 * (P.nx - 1)) / P.se_ax;
-                        const double ey = ((double)i - 0.5 * (P.ny - 1)) / P.se_ay;
-                        if (ex * ex + ey * ey <= 1.0) {
-                            const double dr = (double)P.x[o] - (double)P.se_ref[(size_t)i * P.nx + j];
-                            sse += dr * dr;
-                        }
-                    }
-                }
-            }
-    if (t == 0) P.tilecnt[tile] = 0;   // ready for the next launch
-    if (!(bayes && is_g[0]) && !want_se) return;
-    // the tiles' sums, added in tile order by the last tile to finish: f = r^2 ||R x - b||^2 +
-    // ||x - mu_X||^2, and SE = sqrt(sum over S)
-    const double bs = block_sum<kBwdThreads>(sx, red);
-    const double be = block_sum<kBwdThreads>(sse, red);
-    const int ntiles = (prefix[pi + 1] - prefix[pi]) / parts;
-    if (t == 0) {
-        P.partial[tile] = bs;
-        P.partial[ntiles + tile] = be;
-    }
-    if (last_block(&P.counter[4], ntiles, &last_sh)) {
-        double tot, tse;
-        block_sum_array2<kBwdThreads>(P.partial, P.partial + ntiles, ntiles, red, &tot, &tse);
-        if (t == 0) {
-            Scal *sc = P.sc;
-            if (bayes) {
-                sc->f = P.r2 * sc->f_ls + tot;
-                if (sc->init) sc->f0 = sc->f;
-            }
-            if (want_se) P.se_log[sc->k] = sqrt(tse);   // body sc->k + 1 (k counts finished bodies)
-            P.counter[4] = 0;
-        }
-    }
+    bwd_finish<DUAL, PX>(P, (prefix[pi + 1] - prefix[pi]) / parts, pi, mode, io, parts, vpart, tile, grp, tg, bad != 0, part,
+                         comp, comb, red, &bad_sh, &last_sh, [&](int e, int *i, int *jj) {
+                             *i = i0 + ly + kBwdRowStep * e;
+                             *jj = j;
+                             return *i < P.ny && j < P.nx;
+                         });
 }
 
 // Blocks per problem: `parts` per pixel tile of `ti` rows.
@@ -424,7 +316,8 @@ int backward_blocks(int nx, int ny, int parts, int ti)
 // else to issue.  One R^T y with 32 rows and as chosen, us: 64^2 / 90 views 16.4 and 9.6 (8 rows),
 // 128^2 / 180 20.6 and 14.4 (8), 160^2 / 200 20.6 and 16.4 (16), 192^2 / 240 20.6 and 18.5 (16); from
 // 224^2 / 300 on (28.7) the 32-row grid has more than one block per SM and stays.  The solver's dual pass at 64^2:
-// 25.6 and 14.6.
+// 25.6 and 14.6.  Over mirror pairs, tiles of half the rows (on both sides of the image) by the same rule:
+// 9.6 us at 64^2 (4 rows; 12.3 with 8), the dual pass 14.3 (16.1).
 int bwd_tile_rows(long long blocks32, int nsm)
 {
     return 4 * blocks32 <= 2 * nsm ? 8 : (2 * blocks32 <= 2 * nsm ? 16 : kBwdTileI);

@@ -18,6 +18,8 @@ constexpr int kMaxRadix = 64;        // largest prime factor handled by the gene
 constexpr int kRowsPerChunk = 16;    // forward projector: image rows staged per TMA box
 constexpr int kBwdTileI = 32;        // backprojector pixel tile (rows)
 constexpr int kBwdViewParts = 4;     // backprojector: default blocks per tile (view parts), each a share of the view chunks
+constexpr int kPairTileI = 16;        // backprojector over mirror pairs: tile rows (of 32 columns and their mirror columns)
+constexpr int kPairWindowMax = 88;    // its widest window: two blocks of the solver's pass fit an SM
 constexpr int kBwdMaxParts = 8;      // backprojector: most view parts per tile (supcg_set_bwd_parts)
 constexpr int kBwdTileJ = 32;        // backprojector pixel tile (columns)
 constexpr int kBwdViewChunk = 32;    // backprojector: views staged per shared-memory chunk
@@ -213,6 +215,8 @@ struct Prob {
     float cx, cy, uc;      // uc = (U-1)/2 - off/ds (approximate uses)
     float uc_hi, uc_lo;    // exact split of uc (see ViewP)
     int bwin;              // backprojector: bins staged per view and tile (multiple of 4)
+    int bwp, nbi;          // the same over mirror pairs, and its number of items (0: the general kernel)
+    const int2 *bitems;    // [nbi]: pairs of views (v, mirror of v), then unpaired ones (v, -1)
     const ViewP *views;    // [V]
     const int *vlist;      // [nA + nB]: class-A views, then class-B views
     const int *mirror;     // nullable [V]: the partner of a mirror pair's first view, else -1
@@ -724,7 +728,7 @@ struct Launch {
     int blocks;            // total blocks
     int bw_max;            // widest forward box (floats) among the problems
     int bparts;            // backprojector view parts shared by every problem, 0 if they differ
-    int bwd_ti;            // backprojector tile rows (with the default view parts)
+    int bwd_ti, bwdp_ti;   // backprojector tile rows (with the default view parts): general, over mirror pairs
     int mirror;            // 1: some problem has mirror pairs of views (the forward projector's paired variant)
     cudaStream_t st;
 };
@@ -736,6 +740,8 @@ int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side t
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st);
 int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
 int backward_blocks(int nx, int ny, int parts, int ti);
+int backward_pairs_blocks(int nx, int ny, int parts, int ti);
+int launch_backward_pairs(const Launch &L, bool dual, int mode, int bwp, const Io &io);
 int bwd_tile_rows(long long blocks32, int nsm);   // tile rows of a launch that has blocks32 blocks with 32 rows
 int encode_tiled(CUtensorMap *m, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims,
                  const cuuint64_t *strides_bytes, const cuuint32_t *box);
