@@ -67,6 +67,15 @@ static int encode_map(CUtensorMap *m, float *base, int inner, int outer, int pit
     return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box);
 }
 
+// The same for two arrays of one allocation as the planes of a 3-D map (b above a, both 256-byte aligned).
+static int encode_map2(CUtensorMap *m, float *a, float *b, int inner, int outer, int pitch, int BW, int rows)
+{
+    const cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)outer, 2};
+    const cuuint64_t strides[2] = {(cuuint64_t)pitch * 4, (cuuint64_t)((char *)b - (char *)a)};
+    const cuuint32_t box[3] = {(cuuint32_t)BW, (cuuint32_t)rows, 2};
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a, dims, strides, box);
+}
+
 // ------------------------------------------------------------------ FFT plan
 static int fft_factor(int n, int *rad)
 {
@@ -778,15 +787,15 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.r2 = 0.0;
         P.gray_scale = g->ds / ((double)g->V * g->nx * g->ny * g->d * g->d);
         int e = 0;
-        // 2 w + c: image w (x, p, d) in layout c (rows, transposed); 6 + 2 w + c: its mirror
+        // 2 w + c: image w (x, p, d) in layout c (rows, transposed); 6 + 2 w + c: it and its mirror
         float *imgs[3][2] = {{P.x, P.xT}, {P.p, P.pT}, {P.d, P.dT}};
         float *mimgs[3][2] = {{P.xm, P.xmT}, {P.pm, P.pmT}, {P.dm, P.dmT}};
         for (int wi = 0; wi < 3; ++wi) {
             e |= encode_map(&P.tm[2 * wi], imgs[wi][0], g->nx, g->ny, g->nxp, g->BW, kRowsPerChunk);
             e |= encode_map(&P.tm[2 * wi + 1], imgs[wi][1], g->ny, g->nx, g->nyp, g->BW, kRowsPerChunk);
             if (mir) {
-                e |= encode_map(&P.tm[6 + 2 * wi], mimgs[wi][0], g->nx, g->ny, g->nxp, g->BW, kRowsPerChunk);
-                e |= encode_map(&P.tm[7 + 2 * wi], mimgs[wi][1], g->ny, g->nx, g->nyp, g->BW, kRowsPerChunk);
+                e |= encode_map2(&P.tm[6 + 2 * wi], imgs[wi][0], mimgs[wi][0], g->nx, g->ny, g->nxp, g->BW, kRowsPerChunk);
+                e |= encode_map2(&P.tm[7 + 2 * wi], imgs[wi][1], mimgs[wi][1], g->ny, g->nx, g->nyp, g->BW, kRowsPerChunk);
             }
         }
         if (e) { delete w; return SUPCG_ERR_CUDA; }

@@ -206,7 +206,7 @@ struct Scal {
 struct Prob {
     CUtensorMap tm[12];    // TMA maps (FP32, padded pitches) of the projected images: 2 w + c for image w
                            // (0 = x, 1 = p, 2 = d) in layout c (0 = rows, 1 = transposed); 6 + 2 w + c the
-                           // same of the mirrored images (only with mirror pairs)
+                           // same image and its mirror as two planes (only with mirror pairs)
     int nx, ny, V, U;
     int nxp, nyp, Up;      // pitches in elements: image, transposed image, sinogram
     int BU, BW, ntu;       // forward tiling: bins per tile, box width, bin tiles per view
@@ -688,6 +688,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
 }
 
 // 2-D tiled TMA load of box (x0 = innermost coordinate, y0) into shared memory.
+__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tm, int x0, int y0, int z0, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(x0), "r"(y0), "r"(z0), "r"(smem_u32(bar))
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *tm, int x0, int y0, uint64_t *bar)
 {
     asm volatile(

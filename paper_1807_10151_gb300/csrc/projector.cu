@@ -273,8 +273,8 @@ __device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const C
     auto issue = [&](int slot, int qs, int c) {
         float *dst = proj_dyn + patch0 + slot * buf_elems;
         mbar_expect_tx(&bars[slot], buf_elems * 4);
-        tma_load_2d(dst, tm, qs, c * RC, &bars[slot]);
-        if (MIR) tma_load_2d(dst + moff, tm_m, qs, c * RC, &bars[slot]);
+        if (MIR) tma_load_3d(dst, tm_m, qs, c * RC, 0, &bars[slot]);   // both images in one copy: a copy holds up its warp ~100 cycles
+        else tma_load_2d(dst, tm, qs, c * RC, &bars[slot]);
     };
     int r_lo = n_outer, r_hi = -1;
 #pragma unroll
