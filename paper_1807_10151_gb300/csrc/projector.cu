@@ -10,8 +10,8 @@
 // class A (|cos| >= |sin|) walks image rows, class B walks image columns, and
 // class B reads the transposed image x^T so that both classes walk contiguous
 // rows of the array they read.  Each warp stages chunks of kRowsPerChunk rows
-// x BW columns covering its 64 rays in shared memory by 2-D TMA loads (its own
-// kFwdBufs boxes, one mbarrier each), and only the rows its rays can meet.
+// x BW columns covering its 64 rays in shared memory by TMA loads (its own
+// box and mbarrier), and only the rows its rays can meet.
 // For every row a ray can only cross the two (three near the diagonal)
 // columns nearest to its centre; each is weighted by the shared trapezoid.
 #include "internal.cuh"
@@ -24,7 +24,6 @@ extern __shared__ __align__(128) float proj_dyn[];
 
 static_assert(kRowsPerChunk % 8 == 0, "chunks start at multiples of the fold groups");
 
-constexpr int kFwdBufs = 1;   // forward projector: staged boxes per warp (1: more resident warps hide the copies)
 
 // ============================================================ forward
 // Inner loop over the rows [o0, o0 + rows) of one staged box.  A ray meets a
@@ -231,50 +230,50 @@ __device__ __forceinline__ void fwd_row_terms(const Prob &P, const ViewP &vp, in
     __syncwarp();
 }
 
-// Lower end (multiple of 4) of the inner range that chunk [o0, o0+RC) of the
-// block's rays [u_first, u_last] can touch.
+// Lower end (multiple of 4: the 16-byte rule of a copy) of the inner range that the warp's rays can touch in
+// the chunk of rows from o0 on; b_min: the least centre of its first and last ray at outer index 0.
 template <int RC>
-__device__ __forceinline__ int fwd_box_start(const ViewP &vp, float tf, float tl, int o0)
+__device__ __forceinline__ int fwd_box_start(float b_o, float b_min, int o0)
 {
-    const float bf = __fmaf_rn(vp.a_tau, tf, vp.g0);
-    const float bl = __fmaf_rn(vp.a_tau, tl, vp.g0);
-    const float o_a = __int2float_rn(o0), o_b = __int2float_rn(o0 + RC - 1);
-    float m = fminf(fminf(__fmaf_rn(vp.b_o, o_a, bf), __fmaf_rn(vp.b_o, o_b, bf)),
-                    fminf(__fmaf_rn(vp.b_o, o_a, bl), __fmaf_rn(vp.b_o, o_b, bl)));
-    int lo = __float2int_rd(m) - 3;
-    return lo & ~3;   // round down to a multiple of 4 floats (16-byte TMA rule)
+    return (__float2int_rd(__fmaf_rn(b_o, __int2float_rn(b_o < 0.0f ? o0 + RC - 1 : o0), b_min)) - 3) & ~3;
 }
 
 // Two rays per lane (u and u + 32: 64 consecutive bins per warp); each warp
-// runs its own pipeline of kFwdBufs kRowsPerChunk-row boxes (BW columns
-// covering its 64 rays), so warps never wait for one another.  The warp walks
+// stages its own kRowsPerChunk-row boxes (BW columns covering its 64 rays) in
+// one buffer, so warps never wait for one another.  The warp walks
 // only the chunks holding rows that one of its rays can meet, and within them
 // only those rows.  Rays past the block's last bin follow the last ray (inside
 // the box) and are dropped by the caller.
-// MIR: each chunk also stages the same box of the mirrored image (tm_m) right after the
+// MIR: each chunk's copy also holds the same box of the mirrored image (tm_m: both), after the
 // image's, and acc_m receives the sums of the same bins in the mirror view.
+//
+// Bound by latency and issue at the 14 warps per SM that the boxes leave room for (56 % of the issue slots,
+// shared memory 74 % busy): the work per chunk besides its rows counts.  One copy for both boxes, that work
+// moved in front of the wait for the copy, the next box's position ready when the rows end, and the window
+// check on pairs took R x at 512^2 / 720 views from 121 to 114 us and two of 2048^2 from 10.84 to 10.50 ms.
+// Two half-height boxes per warp, one copied while the other is summed, were slower (146 us), and so were
+// fewer rays per warp without bank conflicts and with narrower boxes (122 us).
 template <bool CLASS_B, bool AXIS, int NC, bool MIR>
 __device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const CUtensorMap *tm, const CUtensorMap *tm_m,
-                                         int patch0, uint64_t *bars, float4 *rtab, int n_outer, int n_inner, int uA,
+                                         int patch0, uint64_t *bar, float4 *rtab, int n_outer, int n_inner, int uA,
                                          int uB, int u_last, float tf, float tl, int *bad, int *timed_out, double *acc,
                                          double *acc_m)
 {
     constexpr int RC = kRowsPerChunk;
     const int BW = P.BW;
     const int box_elems = RC * BW;
-    // one staged chunk: the image's box, then the mirror's
+    // the staged chunk: the image's box, then the mirror's
     const int buf_elems = (MIR ? 2 : 1) * box_elems;
     const int moff = box_elems;
     const int lane = threadIdx.x & 31;
     const int uc[2] = {min(uA, u_last), min(uB, u_last)};
     float tau_hi[2], base[2], sum[2] = {0.0f, 0.0f}, comp[2] = {0.0f, 0.0f};
     float msum[2] = {0.0f, 0.0f}, mcomp[2] = {0.0f, 0.0f};
-    // the chunk's boxes, in their order in the buffer
-    auto issue = [&](int slot, int qs, int c) {
-        float *dst = proj_dyn + patch0 + slot * buf_elems;
-        mbar_expect_tx(&bars[slot], buf_elems * 4);
-        if (MIR) tma_load_3d(dst, tm_m, qs, c * RC, 0, &bars[slot]);   // both images in one copy: a copy holds up its warp ~100 cycles
-        else tma_load_2d(dst, tm, qs, c * RC, &bars[slot]);
+    auto issue = [&](int q0, int c) {   // chunk c's box (MIR: and the mirror's, in the same copy) from inner index q0
+        float *dst = proj_dyn + patch0;
+        mbar_expect_tx(bar, buf_elems * 4);
+        if (MIR) tma_load_3d(dst, tm_m, q0, c * RC, 0, bar);
+        else tma_load_2d(dst, tm, q0, c * RC, bar);
     };
     int r_lo = n_outer, r_hi = -1;
 #pragma unroll
@@ -288,66 +287,56 @@ __device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const C
             r_hi = max(r_hi, hi);
         }
     }
-    const uint64_t tau2 = pk2(tau_hi[0], tau_hi[1]);
+    const uint64_t tau2 = pk2(tau_hi[0], tau_hi[1]), base2 = pk2(base[0], base[1]);
+    const uint64_t bo2 = pk2(vp.b_o, vp.b_o), mag2 = pk2(kCeilMagic, kCeilMagic);
     const int w_lo = __reduce_min_sync(0xffffffffu, r_lo), w_hi = __reduce_max_sync(0xffffffffu, r_hi);
     const int c_first = w_hi >= w_lo ? w_lo / RC : 0;
     const int nch = w_hi >= w_lo ? w_hi / RC - c_first + 1 : 0;   // chunks with at least one of the warp's rows
-    // each box's first inner index, computed once (every lane: the copy and the rows use it)
-    int qs_buf[kFwdBufs];
-#pragma unroll
-    for (int ci = 0; ci < kFwdBufs; ++ci) qs_buf[ci] = fwd_box_start<RC>(vp, tf, tl, (c_first + ci) * RC);
-    if (lane == 0) {
-        for (int ci = 0; ci < kFwdBufs && ci < nch; ++ci) issue(ci, qs_buf[ci], c_first + ci);
-    }
+    const float b_min = fminf(__fmaf_rn(vp.a_tau, tf, vp.g0), __fmaf_rn(vp.a_tau, tl, vp.g0));
+    int qs = fwd_box_start<RC>(vp.b_o, b_min, c_first * RC);   // the box's first inner index
+    if (lane == 0 && nch > 0) issue(qs, c_first);
     for (int ci = 0; ci < nch; ++ci) {
-        const int buf = ci % kFwdBufs, c = c_first + ci;
-        const bool ok = mbar_wait(&bars[buf], (ci / kFwdBufs) & 1);
-        const int o0 = c * RC;
+        // what the chunk needs besides its pixels, and the next box's position, while the copy is on its way
+        const int c = c_first + ci, o0 = c * RC;
         fwd_row_terms<CLASS_B, RC>(P, vp, o0, lane, rtab);
         const int rows = min(RC, n_outer - o0);
         const int rb = max(0, w_lo - o0), re = min(rows, w_hi - o0 + 1);
+        // ray centres at row o0.  The first candidate is monotone in the row: its end values (with
+        // one index of slack for rounding) bound every row of the chunk
+        const uint64_t qm2 = fma2_rn(bo2, pk2(__int2float_rn(o0), __int2float_rn(o0)), base2);
+        const uint64_t qh2 = sub2_rn(qm2, pk2(vp.hwq, vp.hwq)), last2 = pk2(__int2float_rn(rows - 1), __int2float_rn(rows - 1));
+        float q4[4];
+        upk2(add2_rp(qh2, mag2), q4[0], q4[1]);
+        upk2(add2_rp(fma2_rn(last2, bo2, qh2), mag2), q4[2], q4[3]);
+        const bool inside = magic_int(fminf(fminf(q4[0], q4[1]), fminf(q4[2], q4[3]))) >= qs + 1 &&
+                            magic_int(fmaxf(fmaxf(q4[0], q4[1]), fmaxf(q4[2], q4[3]))) <= qs + BW - NC - 1;
+        const int qs_next = fwd_box_start<RC>(vp.b_o, b_min, o0 + RC);
+        const bool ok = mbar_wait(bar, ci & 1);
         if (ok && rb < re) {
-            const int qs = qs_buf[buf];
-            float qm[2];
-            bool inside = true;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                qm[q] = __fmaf_rn(vp.b_o, __int2float_rn(o0), base[q]);   // ray centre at row o0
-                // the first candidate is monotone in the row: its end values (with one index
-                // of slack for rounding) bound every row of the chunk
-                const float qh = __fsub_rn(qm[q], vp.hwq);
-                const int qa = __float2int_ru(qh) - qs;
-                const int qb = __float2int_ru(__fmaf_rn((float)(rows - 1), vp.b_o, qh)) - qs;
-                inside = inside && min(qa, qb) >= 1 && max(qa, qb) <= BW - NC - 1;
-            }
-            const int pb = patch0 + buf * buf_elems;
             // axis-aligned views too: every ray of theirs crosses every row, so that on the
             // scalar path their items were the longest of a pass (108-118 us against a mean
             // of 47 us at 512^2 / 720 views) and set its length
             if (inside) {
-                fwd_rows2<CLASS_B, AXIS, NC, MIR>(P, vp, tau2, pk2(qm[0], qm[1]), o0, rb, re, qs, pb, moff, rtab, sum,
+                fwd_rows2<CLASS_B, AXIS, NC, MIR>(P, vp, tau2, qm2, o0, rb, re, qs, patch0, moff, rtab, sum,
                                                   comp, msum, mcomp);
             } else {
+                float qm[2];
+                upk2(qm2, qm[0], qm[1]);
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
-                    fwd_rows<CLASS_B, AXIS, NC, true, MIR>(P, vp, tau_hi[q], qm[q], o0, rb, re, qs, pb, moff, bad, sum[q],
-                                                           comp[q], msum[q], mcomp[q]);
+                    fwd_rows<CLASS_B, AXIS, NC, true, MIR>(P, vp, tau_hi[q], qm[q], o0, rb, re, qs, patch0, moff, bad,
+                                                           sum[q], comp[q], msum[q], mcomp[q]);
             }
         }
-        // every lane is done with this buffer; a timeout in any lane ends the warp's loop
+        // every lane is done with the buffer; a timeout in any lane ends the warp's loop
         if (__any_sync(0xffffffffu, !ok)) {
             *timed_out = 1;
-            if (lane == 0) {   // bounded waits for the copies still in flight: chunk ci's and, if issued, ci + 1's
-                for (int cj = ci; cj < ci + kFwdBufs && cj < nch; ++cj)   // this chunk and those issued after it
-                    (void)mbar_wait(&bars[cj % kFwdBufs], (cj / kFwdBufs) & 1);
-            }
+            if (lane == 0) (void)mbar_wait(bar, ci & 1);   // a bounded wait for the copy still in flight
             break;
         }
         __syncwarp();
-        if (ci + kFwdBufs < nch) {
-            qs_buf[buf] = fwd_box_start<RC>(vp, tf, tl, (c + kFwdBufs) * RC);
-            if (lane == 0) issue(buf, qs_buf[buf], c + kFwdBufs);
-        }
+        if (lane == 0 && ci + 1 < nch) issue(qs_next, c + 1);
+        qs = qs_next;
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {   // weights in units of P
@@ -367,8 +356,8 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
                                                                         const int *__restrict__ prefix, int count,
                                                                         int which, int mode, Io io)
 {
-    // proj_dyn: [warp][kFwdBufs][box: the image, (MIRK) its mirror][kRowsPerChunk][BW]
-    __shared__ __align__(8) uint64_t bars[kFwdBufs * (kFwdThreads / 32)];   // one per staged box
+    // proj_dyn: [warp][box: the image, (MIRK) its mirror][kRowsPerChunk][BW]
+    __shared__ __align__(8) uint64_t bars[kFwdThreads / 32];               // one per warp
     __shared__ float4 rowtab[kFwdThreads / 32][kRowsPerChunk];             // each warp's row terms
     __shared__ __align__(16) double red[40];
     __shared__ int flag;
@@ -399,8 +388,8 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
     const CUtensorMap *tm = &P.tm[which * 2 + cb];
     const CUtensorMap *tm_m = &P.tm[6 + which * 2 + cb];
     // this warp's boxes in proj_dyn
-    const int patch0 = warp * kFwdBufs * (MIRK ? 2 : 1) * kRowsPerChunk * P.BW;
-    uint64_t *wbars = bars + kFwdBufs * warp;
+    const int patch0 = warp * (MIRK ? 2 : 1) * kRowsPerChunk * P.BW;
+    uint64_t *wbars = bars + warp;
 
     const int u_first = tile * P.BU;
     const int u_last = min(P.U, u_first + P.BU) - 1;
@@ -410,7 +399,7 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
     const float tf = bin_pos(min(uw0, u_last), P.uc), tl = bin_pos(uw1, P.uc);
 
     if (t == 0) bad_sh = 0;
-    if (t < kFwdBufs * (kFwdThreads / 32)) mbar_init(&bars[t], 1);
+    if (t < kFwdThreads / 32) mbar_init(&bars[t], 1);
     if (t == 0) fence_mbar_init();
     __syncthreads();
 
@@ -539,9 +528,8 @@ static int launch_forward_t(const Launch &L, int which, int mode, const Io &io)
     // every problem's BW <= 256, so the warps' box buffers never exceed this size; with mirror
     // pairs each chunk holds two boxes
     constexpr int rows = (MIRK ? 2 : 1) * kRowsPerChunk;
-    const int per_warp = kFwdBufs * rows;
-    const int smem = (kFwdThreads / 32) * per_warp * L.bw_max * 4;
-    int rc = func_attrs_once((const void *)k_forward<MIRK>, (kFwdThreads / 32) * per_warp * 256 * 4);
+    const int smem = (kFwdThreads / 32) * rows * L.bw_max * 4;
+    int rc = func_attrs_once((const void *)k_forward<MIRK>, (kFwdThreads / 32) * rows * 256 * 4);
     if (rc) return rc;
     k_forward<MIRK><<<L.blocks, kFwdThreads, smem, L.st>>>(L.probs, L.prefix, L.count, which, mode, io);
     SUPCG_CUDA_TRY(cudaGetLastError());
