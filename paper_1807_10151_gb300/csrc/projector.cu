@@ -37,22 +37,23 @@ static_assert(kRowsPerChunk % 8 == 0, "chunks start at multiples of the fold gro
 // MIR: the staged box is followed (moff floats later) by the same box of the
 // left-right mirrored image; each weight is also applied there, giving the ray
 // of the same bin in the mirror view (msum, mcomp: its compensated sum).
-template <bool CLASS_B, bool AXIS, int NC, bool CHECKED, bool MIR>
+template <bool AXIS, int NC, bool CHECKED, bool MIR>
 __device__ __forceinline__ void fwd_rows(const Prob &P, const ViewP &vp, float tau_hi, float qm, int o0, int rb,
                                          int re, int qs, int pbase, int moff, int *bad,
                                          float &sum, float &comp, float &msum, float &mcomp)
 {
     const int BW = P.BW;
+    const bool cb = (vp.flags & kViewClassB) != 0;
     // outer coordinate of row o0 + rb (pixel units) and its change per row
-    float Oc = CLASS_B ? __fsub_rn(__int2float_rn(o0 + rb), P.cx) : __fsub_rn(P.cy, __int2float_rn(o0 + rb));
-    const float dO = CLASS_B ? 1.0f : -1.0f;
-    const float hi_o = CLASS_B ? vp.cu_hi : vp.su_hi;   // coefficient of the outer coordinate
-    const float lo_o = CLASS_B ? vp.cu_lo : vp.su_lo;
-    const float hi_i = CLASS_B ? vp.su_hi : vp.cu_hi;   // coefficient of the inner coordinate
-    const float lo_i = CLASS_B ? vp.su_lo : vp.cu_lo;
+    float Oc = cb ? __fsub_rn(__int2float_rn(o0 + rb), P.cx) : __fsub_rn(P.cy, __int2float_rn(o0 + rb));
+    const float dO = cb ? 1.0f : -1.0f;
+    const float hi_o = cb ? vp.cu_hi : vp.su_hi;   // coefficient of the outer coordinate
+    const float lo_o = cb ? vp.cu_lo : vp.su_lo;
+    const float hi_i = cb ? vp.su_hi : vp.cu_hi;   // coefficient of the inner coordinate
+    const float lo_i = cb ? vp.su_lo : vp.cu_lo;
     // inner coordinate of inner index q: X = q - cx (class A) or Y = cy - q (class B)
-    const float c_in = CLASS_B ? P.cy : P.cx;
-    const float dI = CLASS_B ? -1.0f : 1.0f;
+    const float c_in = cb ? P.cy : P.cx;
+    const float dI = cb ? -1.0f : 1.0f;
     const float E = vp.E, Sn = vp.Sn, ESn = vp.ESn;
     const float qh = __fsub_rn(qm, vp.hwq);
     const int prow = pbase - qs;   // proj_dyn index of inner index 0 of the box's first row
@@ -73,7 +74,7 @@ __device__ __forceinline__ void fwd_rows(const Prob &P, const ViewP &vp, float t
         const float rsmall = __fmaf_rn(lo_o, Oc, P.uc_lo);
         Oc = __fadd_rn(Oc, dO);
         const float q0f = CHECKED ? __int2float_rn(q0) : magic_float(qc);   // the clamped index when checked
-        const float I0 = CLASS_B ? __fsub_rn(c_in, q0f) : __fsub_rn(q0f, c_in);
+        const float I0 = cb ? __fsub_rn(c_in, q0f) : __fsub_rn(q0f, c_in);
         float I = I0;
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
@@ -123,22 +124,36 @@ __device__ __forceinline__ void fwd_rows(const Prob &P, const ViewP &vp, float t
     }
 }
 
+// A view's coefficients by the walked direction.  The inner coordinate is I = q - cx (class A) or cy - q (B), the
+// outer one O = cy - o (A) or o - cx (B); with the signs in the coefficients (exact) both are index minus centre, so
+// that one copy of the code serves both classes: half the instructions to hold in the caches when an SM's
+// warps are in views of both.  R x at 512^2 / 720 views 115.5 -> 110.8 us, a solve there 4.31 -> 4.11 ms.
+struct FwdClass {
+    float hi_i, lo_i, c_in, hi_o, lo_o, c_out;
+    __device__ __forceinline__ FwdClass(const Prob &P, const ViewP &vp)
+    {
+        const bool cb = (vp.flags & kViewClassB) != 0;
+        hi_i = cb ? -vp.su_hi : vp.cu_hi;
+        lo_i = cb ? -vp.su_lo : vp.cu_lo;
+        hi_o = cb ? vp.cu_hi : -vp.su_hi;
+        lo_o = cb ? vp.cu_lo : -vp.su_lo;
+        c_in = cb ? P.cy : P.cx;
+        c_out = cb ? P.cx : P.cy;
+    }
+};
+
 // Two rays per lane (A, B), every per-ray FP32 step as one f32x2 instruction
 // for both: the candidate index, the exact-split coordinates and each
 // candidate's weight (lane for lane the scalar IEEE steps of fwd_rows, so
 // the weights are the same bits).  Only for boxes that hold every candidate.
-template <bool CLASS_B, bool AXIS, int NC, bool MIR>
-__device__ __forceinline__ void fwd_rows2(const Prob &P, const ViewP &vp, uint64_t tau2, uint64_t qm2, int o0, int rb,
+template <bool AXIS, int NC, bool MIR>
+__device__ __forceinline__ void fwd_rows2(const Prob &P, const ViewP &vp, const FwdClass &c, uint64_t tau2, uint64_t qm2, int o0, int rb,
                                           int re, int qs, int pbase, int moff, const float4 *rtab,
                                           float *sum, float *comp, float *msum, float *mcomp)
 {
     const int BW = P.BW;
-    const float hi_i = CLASS_B ? vp.su_hi : vp.cu_hi;   // coefficient of the inner coordinate
-    const float lo_i = CLASS_B ? vp.su_lo : vp.cu_lo;
-    const float c_in = CLASS_B ? P.cy : P.cx;           // inner coordinate = q - cx (A) or cy - q (B)
-    const float dI = CLASS_B ? -1.0f : 1.0f;
     const float E = vp.E, Sn = vp.Sn, ESn = vp.ESn;
-    const uint64_t hii2 = pk2(-hi_i, -hi_i), loi2 = pk2(lo_i, lo_i), cin2 = pk2(c_in, c_in), dI2 = pk2(dI, dI);
+    const uint64_t hii2 = pk2(-c.hi_i, -c.hi_i), loi2 = pk2(c.lo_i, c.lo_i), cin2 = pk2(c.c_in, c.c_in);
     const uint64_t bo2 = pk2(vp.b_o, vp.b_o), mag2 = pk2(kCeilMagic, kCeilMagic);
     const uint64_t qh2 = sub2_rn(qm2, pk2(vp.hwq, vp.hwq));
     const int prow = pbase - qs;   // proj_dyn index of inner index 0 of the box's first row
@@ -154,10 +169,10 @@ __device__ __forceinline__ void fwd_rows2(const Prob &P, const ViewP &vp, uint64
         const uint64_t rbig2 = add2_rn(tau2, pk2(rt.x, rt.y));       // exact
         const uint64_t rsmall2 = pk2(rt.z, rt.w);
         const uint64_t q0f2 = sub2_rn(qc2, mag2);
-        uint64_t I2 = CLASS_B ? sub2_rn(cin2, q0f2) : sub2_rn(q0f2, cin2);   // exact half-integers
+        uint64_t I2 = sub2_rn(q0f2, cin2);   // exact half-integers
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
-            if (k) I2 = add2_rn(I2, dI2);
+            if (k) I2 = add2_rn(I2, pk2(1.0f, 1.0f));
             const uint64_t big2 = fma2_rn(hii2, I2, rbig2);          // exact
             float dA, dB;
             upk2(sub2_rn(big2, fma2_rn(loi2, I2, rsmall2)), dA, dB);
@@ -218,13 +233,13 @@ __device__ __forceinline__ void fwd_rows2(const Prob &P, const ViewP &vp, uint64
 // and s = lo_o O + uc_lo (rounded once), O the outer coordinate of row o0 + r, so that
 // a ray's row needs big = tau_hi + H (exact, the value of fma(-hi_o, O, tau_hi)) and s.
 // Written by lanes 0 .. RC-1 of the warp that reads it.
-template <bool CLASS_B, int RC>
-__device__ __forceinline__ void fwd_row_terms(const Prob &P, const ViewP &vp, int o0, int lane, float4 *rtab)
+template <int RC>
+__device__ __forceinline__ void fwd_row_terms(const FwdClass &c, float uc_lo, int o0, int lane, float4 *rtab)
 {
     if (lane < RC) {
-        const float O = CLASS_B ? __fsub_rn(__int2float_rn(o0 + lane), P.cx) : __fsub_rn(P.cy, __int2float_rn(o0 + lane));
-        const float H = __fmul_rn(CLASS_B ? -vp.cu_hi : -vp.su_hi, O);
-        const float sm = __fmaf_rn(CLASS_B ? vp.cu_lo : vp.su_lo, O, P.uc_lo);
+        const float O = __fsub_rn(__int2float_rn(o0 + lane), c.c_out);
+        const float H = __fmul_rn(-c.hi_o, O);
+        const float sm = __fmaf_rn(c.lo_o, O, uc_lo);
         rtab[lane] = make_float4(H, H, sm, sm);
     }
     __syncwarp();
@@ -253,13 +268,14 @@ __device__ __forceinline__ int fwd_box_start(float b_o, float b_min, int o0)
 // check on pairs took R x at 512^2 / 720 views from 121 to 114 us and two of 2048^2 from 10.84 to 10.50 ms.
 // Two half-height boxes per warp, one copied while the other is summed, were slower (146 us), and so were
 // fewer rays per warp without bank conflicts and with narrower boxes (122 us).
-template <bool CLASS_B, bool AXIS, int NC, bool MIR>
-__device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const CUtensorMap *tm, const CUtensorMap *tm_m,
+template <bool AXIS, int NC, bool MIR>
+__device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const ViewP *vg, const CUtensorMap *tm, const CUtensorMap *tm_m,
                                          int patch0, uint64_t *bar, float4 *rtab, int n_outer, int n_inner, int uA,
                                          int uB, int u_last, float tf, float tl, int *bad, int *timed_out, double *acc,
                                          double *acc_m)
 {
     constexpr int RC = kRowsPerChunk;
+    const FwdClass fc(P, vp);
     const int BW = P.BW;
     const int box_elems = RC * BW;
     // the staged chunk: the image's box, then the mirror's
@@ -298,7 +314,7 @@ __device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const C
     for (int ci = 0; ci < nch; ++ci) {
         // what the chunk needs besides its pixels, and the next box's position, while the copy is on its way
         const int c = c_first + ci, o0 = c * RC;
-        fwd_row_terms<CLASS_B, RC>(P, vp, o0, lane, rtab);
+        fwd_row_terms<RC>(fc, P.uc_lo, o0, lane, rtab);
         const int rows = min(RC, n_outer - o0);
         const int rb = max(0, w_lo - o0), re = min(rows, w_hi - o0 + 1);
         // ray centres at row o0.  The first candidate is monotone in the row: its end values (with
@@ -317,14 +333,14 @@ __device__ __forceinline__ void fwd_ray2(const Prob &P, const ViewP &vp, const C
             // scalar path their items were the longest of a pass (108-118 us against a mean
             // of 47 us at 512^2 / 720 views) and set its length
             if (inside) {
-                fwd_rows2<CLASS_B, AXIS, NC, MIR>(P, vp, tau2, qm2, o0, rb, re, qs, patch0, moff, rtab, sum,
+                fwd_rows2<AXIS, NC, MIR>(P, vp, fc, tau2, qm2, o0, rb, re, qs, patch0, moff, rtab, sum,
                                                   comp, msum, mcomp);
             } else {
                 float qm[2];
                 upk2(qm2, qm[0], qm[1]);
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
-                    fwd_rows<CLASS_B, AXIS, NC, true, MIR>(P, vp, tau_hi[q], qm[q], o0, rb, re, qs, patch0, moff, bad,
+                    fwd_rows<AXIS, NC, true, MIR>(P, *vg, tau_hi[q], qm[q], o0, rb, re, qs, patch0, moff, bad,
                                                            sum[q], comp[q], msum[q], mcomp[q]);
             }
         }
@@ -408,21 +424,15 @@ __global__ void __launch_bounds__(kFwdThreads, MIRK ? 7 : 10) k_forward(const Pr
     double acc[2] = {0.0, 0.0}, acc_m[2] = {0.0, 0.0};
     // axis-aligned views meet at most two pixels per row; near-diagonal ones up to three
     const bool three = (vp.flags & kViewFwd3) != 0;
-#define SUPCG_FWD(CB, AX, NC, MIR) \
-    fwd_ray2<CB, AX, NC, MIR>(P, vp, tm, tm_m, patch0, wbars, rowtab[warp], n_outer, n_inner, uA, uB, u_last, tf, tl, \
-                              &bad, &timed_out, acc, acc_m)
+#define SUPCG_FWD(AX, NC, MIR) \
+    fwd_ray2<AX, NC, MIR>(P, vp, &P.views[v], tm, tm_m, patch0, wbars, rowtab[warp], n_outer, n_inner, uA, uB, u_last, tf, tl, &bad, \
+                          &timed_out, acc, acc_m)
     if (idle) {
         // no item for this warp
     } else if (MIRK && vm >= 0) {   // a pair (never axis-aligned: those have no mirror partner)
-        if (classB) {
-            if (three) SUPCG_FWD(true, false, 3, true); else SUPCG_FWD(true, false, 2, true);
-        } else {
-            if (three) SUPCG_FWD(false, false, 3, true); else SUPCG_FWD(false, false, 2, true);
-        }
-    } else if (classB) {
-        if (axis) SUPCG_FWD(true, true, 2, false); else if (three) SUPCG_FWD(true, false, 3, false); else SUPCG_FWD(true, false, 2, false);
+        if (three) SUPCG_FWD(false, 3, true); else SUPCG_FWD(false, 2, true);
     } else {
-        if (axis) SUPCG_FWD(false, true, 2, false); else if (three) SUPCG_FWD(false, false, 3, false); else SUPCG_FWD(false, false, 2, false);
+        if (axis) SUPCG_FWD(true, 2, false); else if (three) SUPCG_FWD(false, 3, false); else SUPCG_FWD(false, 2, false);
     }
 #undef SUPCG_FWD
     if (__syncthreads_or(timed_out)) {   // a warp's copy did not arrive: the whole block leaves
