@@ -47,6 +47,21 @@ def test_solver_pass_changes_no_bit():
         assert torch.equal(xs[c], x) and rep["f_last"] == reps[c]["f_last"]
 
 
+def test_batch_mixing_both_kernels_equals_single_solves():
+    """Problems with and without mirror pairs in one schedule: each kernel's launch skips the other's problems."""
+    import paper_1807_10151_gb300 as S
+    kw = dict(K=1, a=0.99, gamma=0.3, mu=1e-4, rho=0.8, max_iter=5)
+    ogs = [O.Geometry(n, ny=n + 3, V=V, U=U, theta=np.arange(V) * math.pi / V + skew)
+           for n, V, U, skew in ((40, 33, 61, 0.01), (37, 35, 59, 0.0), (70, 20, 101, 0.0), (33, 21, 55, 0.02), (20, 30, 33, 0.0))]
+    g = torch.Generator(device="cuda").manual_seed(6)
+    bs = [torch.rand(og.V, og.U, device="cuda", generator=g) for og in ogs]
+    xs = [torch.zeros(og.ny, og.nx, device="cuda") for og in ogs]
+    reps = S.solve_batched([gpu_geometry(og) for og in ogs], bs, xs, **kw)
+    for og, b, xb, rb in zip(ogs, bs, xs, reps):
+        x, rep, _ = gpu_geometry(og).solve(b, **kw)
+        assert torch.equal(xb, x) and rep["f_last"] == rb["f_last"]
+
+
 # odd and even widths down to one column, half widths at and around a tile's 32 columns, bins finer (three
 # candidates) and coarser than pixels, a shifted detector, and unpaired views among the pairs
 @pytest.mark.parametrize("nx,ny,V,U,off,dsf,extra", [
