@@ -405,7 +405,7 @@ def run_art(args, dev):
     line = {
         "metric": "ART cycles/s (Bayesian criterion, Sec. 3.4)", "value": cycles / t_art, "unit": "cycles/s",
         "n_gpus": 1, "steps": cycles, "warmup": args.warmup, "ms_per_step": 1000.0 * t_art / cycles,
-        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32 (ray sums f64)",
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32 (ray sums double-float)",
         "data": "synthetic",
         "config": {"workload": "art_512x512_720views_725bins_poisson1e5", "art": art_kw, "supart": sup_kw,
                    "class_barriers_per_cycle": WL["V"] * 2, "l2": "the 14 MB working set stays L2-resident"},
