@@ -938,14 +938,11 @@ extern "C" int supcg_project(supcg_geometry g, const void *d_x, void *d_y, int b
     return launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_PLAIN, io);
 }
 
-// R^T y (dual: g from r and h from q in one pass): the problems with mirror pairs, then the others, each if any.
-static int enqueue_backward(Workspace *w, cudaStream_t st, bool dual, int mode, const Io &io)
+// R^T y of the caller's sinograms: one geometry's problems, so one of the two kernels.
+static int enqueue_backproject(Workspace *w, cudaStream_t st, const Io &io)
 {
-    int rc = SUPCG_OK;
-    if (w->blocks[KT_BWDP]) rc = launch_backward_pairs(w->L(KT_BWDP, st), dual, mode, w->bwp, io);
-    if (!rc && w->blocks[KT_BWD])
-        rc = dual ? launch_backward2(w->L(KT_BWD, st), w->bwin) : launch_backward(w->L(KT_BWD, st), mode, w->bwin, io);
-    return rc;
+    return w->blocks[KT_BWDP] ? launch_backward_pairs(w->L(KT_BWDP, st), false, BWD_PLAIN, w->bwp, io)
+                              : launch_backward(w->L(KT_BWD, st), BWD_PLAIN, w->bwin, io);
 }
 
 extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, int batch, void *stream)
@@ -961,10 +958,10 @@ extern "C" int supcg_backproject(supcg_geometry g, const void *d_y, void *d_x, i
     if (scope.rc) return scope.rc;
     // straight into the caller's image, unless it overlaps the sinogram still being read
     const char *y = (const char *)d_y, *x = (const char *)d_x;
-    if (y + batch * m * es <= x || x + batch * n * es <= y) return enqueue_backward(w, st, false, BWD_PLAIN, io);
+    if (y + batch * m * es <= x || x + batch * n * es <= y) return enqueue_backproject(w, st, io);
     Io to_g = io;
     to_g.out = nullptr;
-    if ((rc = enqueue_backward(w, st, false, BWD_PLAIN, to_g))) return rc;
+    if ((rc = enqueue_backproject(w, st, to_g))) return rc;
     return launch_store_out(w->L(KT_VEC, st), 2, io);
 }
 
@@ -1229,7 +1226,8 @@ static int enqueue_body(Workspace *w, const supcg_params *p, cudaStream_t st, in
     }
     // g = R^T r, and h = R^T q of the previous step (A p for this step's beta; the previous alpha
     // took p^T A p from ||q||^2), one pass over the views for both
-    LAUNCH(SUPCG_KIND_BACKWARD, st, enqueue_backward(w, st, true, BWD_G, Io()));
+    if (w->blocks[KT_BWDP]) LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward_pairs(w->L(KT_BWDP, st), true, BWD_G, w->bwp, Io()));
+    if (w->blocks[KT_BWD]) LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward2(w->L(KT_BWD, st), w->bwin));
     if (p->precondition) {                                                      // z = M g; its last pass
         if ((rc = enqueue_precond_k(w, st))) return rc;                         // also forms beta
     } else {
@@ -1246,7 +1244,8 @@ static int enqueue_init(Workspace *w, const supcg_params *p, cudaStream_t st)
 {
     int rc;
     LAUNCH(SUPCG_KIND_FORWARD, st, launch_forward(w->L(KT_FWD, st), w->L(KT_FWDA, st), 0, FWD_RESID));
-    LAUNCH(SUPCG_KIND_BACKWARD, st, enqueue_backward(w, st, false, BWD_G, Io()));
+    if (w->blocks[KT_BWDP]) LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward_pairs(w->L(KT_BWDP, st), false, BWD_G, w->bwp, Io()));
+    if (w->blocks[KT_BWD]) LAUNCH(SUPCG_KIND_BACKWARD, st, launch_backward(w->L(KT_BWD, st), BWD_G, w->bwin));
     if (p->precondition) {
         if ((rc = enqueue_precond_k(w, st))) return rc;
     } else {
