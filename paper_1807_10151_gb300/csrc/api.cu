@@ -863,7 +863,9 @@ static int ws_upload(Workspace *w, cudaStream_t st)
 }
 
 // A standalone operator's work on the workspace: after the last such call's, whatever stream that was on (the
-// scratch is shared), with the descriptors up to date; its end is marked when the call returns.
+// scratch is shared), with the descriptors up to date; its end is marked when the call returns.  A call that is
+// refused here has enqueued nothing and leaves the mark where it was: on a stream under capture it would become
+// a node of that capture, and every later call would be refused for waiting on it.
 struct OpsScope {
     Workspace *w;
     cudaStream_t st;
@@ -877,7 +879,10 @@ struct OpsScope {
             rc = ws_upload(w, st);
         }
     }
-    ~OpsScope() { (void)cudaEventRecord(w->last, st); }
+    ~OpsScope()
+    {
+        if (rc == SUPCG_OK) (void)cudaEventRecord(w->last, st);
+    }
     OpsScope(const OpsScope &) = delete;
     OpsScope &operator=(const OpsScope &) = delete;
 };
