@@ -118,16 +118,12 @@ struct PixWalk {
     }
 };
 
-// Root of the TV term based at (i, j) of y~ = y + c tbar (term must exist).
-__device__ __forceinline__ float trial_term(const float *__restrict__ y, const float *__restrict__ t, int ld,
-                                            int i, int j, float c)
+// The FP32 image value of y + c t, as x_step stores it: from the pair (y, lo) where has_lo.  (k_stv's trials once
+// took the high part's FMA alone, an ulp off the image that an accepted trial leaves and that k_stv_tile's trials
+// take; the pair costs 5 % of K = 40 at 1400^2 and 8 % at 2048^2, 1764 -> 1862 and 2910 -> 3160 us.)
+__device__ __forceinline__ float step_value(float y, float lo, bool has_lo, float c, float t)
 {
-    const size_t p = (size_t)i * ld + j;
-    const float yc = __fmaf_rn(c, t[p], y[p]);
-    const float yd = __fmaf_rn(c, t[p + ld], y[p + ld]);
-    const float yr = __fmaf_rn(c, t[p + 1], y[p + 1]);
-    const float a = yc - yd, b = yc - yr;
-    return sqrtf(a * a + b * b);
+    return has_lo ? df_add(df{y, lo}, df_prod(c, t)).h : __fmaf_rn(c, t, y);
 }
 
 // y <- y + c t at element p of the iterate: in double-float arithmetic on the pair
@@ -484,7 +480,7 @@ __global__ void __launch_bounds__(kTvThreads, 3) k_stv(const Prob *__restrict__ 
             ++trials;
             df s = df_make(0.0f);
             for (PixWalk w(e0, stride, nx); w.i < ny;) {
-                float yv[kStvGroup][3], tv[kStvGroup][3];
+                float yv[kStvGroup][3], lv[kStvGroup][3], tv[kStvGroup][3];
                 bool in[kStvGroup];
 #pragma unroll
                 for (int q = 0; q < kStvGroup; ++q) {
@@ -497,17 +493,21 @@ __global__ void __launch_bounds__(kTvThreads, 3) k_stv(const Prob *__restrict__ 
                         tv[q][0] = tb[p];
                         tv[q][1] = tb[p + ld];
                         tv[q][2] = tb[p + 1];
+                        if (xl) {
+                            lv[q][0] = xl[p];
+                            lv[q][1] = xl[p + ld];
+                            lv[q][2] = xl[p + 1];
+                        }
                     }
                     w.next();
                 }
 #pragma unroll
                 for (int q = 0; q < kStvGroup; ++q) {
                     if (in[q]) {   // the root of the TV term of y~ = y + c tbar based at the pixel
-                        const float yc = __fmaf_rn(c, tv[q][0], yv[q][0]);
-                        const float yd = __fmaf_rn(c, tv[q][1], yv[q][1]);
-                        const float yr = __fmaf_rn(c, tv[q][2], yv[q][2]);
-                        const float a1 = yc - yd, b1 = yc - yr;
-                        df_acc(s, sqrtf(a1 * a1 + b1 * b1));
+                        float y3[3];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) y3[k] = step_value(yv[q][k], xl ? lv[q][k] : 0.0f, xl != nullptr, c, tv[q][k]);
+                        df_acc(s, root(y3[0] - y3[1], y3[0] - y3[2]));
                     }
                 }
             }
@@ -585,9 +585,9 @@ __global__ void __launch_bounds__(kTvThreads, 3) k_stv(const Prob *__restrict__ 
 // block may still be reading one trial's while another writes the next one's.  x is
 // written only at the end.
 //   A TV term's roots and quotients are computed once, at its base pixel, and meet the
-// pixels below and to the right of it in shared memory.  The values are those of
-// k_stv bit for bit, and so are the steps, as long as the two kernels' sums round to
-// the same FP32 step length.
+// pixels below and to the right of it in shared memory.  A pixel's values (y~, its
+// term, tbar) are those of k_stv bit for bit: which kernel a problem takes depends on
+// the other problems of its launch.  The two add up the same terms in another order.
 // Measured, K = 40 at 512^2 (one call): 867 -> 364 us, 6.6 us per step; a grid barrier is
 // about 1.4 us of it, the FP64 sum over the blocks' partials 1 us.
 constexpr int kStvThreads = 512, kStvWarps = kStvThreads / 32;

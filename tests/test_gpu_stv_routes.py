@@ -1,0 +1,36 @@
+"""S_TV by its two kernels: on tiles resident in shared memory where the launch's images fit the
+device, in memory where they do not.  Which one a problem takes depends on how many problems share
+its launch, so both have to give it the same steps."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1807_10151_gb300 import synth
+
+from gpu_cases import gpu_geometry, to_dev
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("K,a,gamma", [(1, 0.995, 0.5), (4, 0.99, 0.05)])
+def test_a_problem_alone_equals_it_in_a_batch_that_does_not_fit(K, a, gamma):
+    """26 images of 243^2 have 416 tiles of 128 rows, more than the device holds at two blocks per SM.
+    l and the image are the same; TV(x_{k-1/2}) is the same terms added in another order: double-float
+    sums of at most 40 terms (2^-47 each), then FP64, so within 1e-12."""
+    import paper_1807_10151_gb300 as S
+    og = O.Geometry(243, V=48, U=345)
+    R = O.CSR(og)
+    bs = [to_dev(np.asarray(synth.gaussian_noise(R.project(synth.ellipse_phantom(243, 12, 700 + c)), 0.01, 800 + c),
+                            np.float32)) for c in range(2)]
+    G = gpu_geometry(og)
+    kw = dict(K=K, a=a, gamma=gamma, mu=1e-5, rho=0.8, max_iter=6)
+    single = [G.solve(b, **kw) for b in bs]
+    n = 26
+    xs = [torch.zeros(243, 243, device="cuda") for _ in range(n)]
+    reps = S.solve_batched([G] * n, [bs[c % 2] for c in range(n)], xs, **kw)
+    for c in (0, 1, n - 1):
+        x1, r1, _ = single[c % 2]
+        assert reps[c]["status"] == 0 and reps[c]["ell"] == r1["ell"]
+        assert reps[c]["tv_last"] == pytest.approx(r1["tv_last"], rel=1e-12, abs=0.0)
+        np.testing.assert_array_equal(xs[c].cpu().numpy(), x1.cpu().numpy())
