@@ -616,14 +616,6 @@ __device__ __forceinline__ void stv_ring(int k, int &i, int &j)
     j = (k & 1) ? S::W - 1 : 0;
 }
 
-// x / T for y = 1 / T correctly rounded: Markstein's quotient (IBM J. Res. Dev. 34, 1990), correctly rounded
-// as the division itself is where x - q T is a normal number or 0.
-__device__ __forceinline__ float quotient(float x, float T, float y)
-{
-    const float q = __fmul_rn(x, y);
-    return __fmaf_rn(__fmaf_rn(-q, T, x), y, q);
-}
-
 // The step scalars of one thread.  An FP64 instruction holds the SM's FP64 pipe for about 38 cycles per warp
 // that issues it; inlined, these were turned into predicated code that every warp issued (350 FP64
 // instructions per step and block, the pipe 85 % busy: 456 us for 40 steps at 512^2 against 364).
@@ -736,10 +728,9 @@ __global__ void __launch_bounds__(kStvThreads, 2) k_stv_tile(const Prob *__restr
                 } else {
                     const float Tl = root_b(a1, b1);
                     T = root(a1, b1);
-                    const float iv = __frcp_rn(T);
-                    va = quotient(a1, T, iv);
-                    vb = quotient(b1, Tl, __frcp_rn(Tl));
-                    vs = quotient(__fadd_rn(a1, b1), T, iv);
+                    va = __fdiv_rn(a1, T);
+                    vb = __fdiv_rn(b1, Tl);
+                    vs = __fdiv_rn(__fadd_rn(a1, b1), T);
                 }
             }
             sm.qa[q] = va;

@@ -34,3 +34,27 @@ def test_a_problem_alone_equals_it_in_a_batch_that_does_not_fit(K, a, gamma):
         assert reps[c]["status"] == 0 and reps[c]["ell"] == r1["ell"]
         assert reps[c]["tv_last"] == pytest.approx(r1["tv_last"], rel=1e-12, abs=0.0)
         np.testing.assert_array_equal(xs[c].cpu().numpy(), x1.cpu().numpy())
+
+
+def test_one_step_on_an_image_whose_quotients_underflow():
+    """The last row's tbar is a / T of the terms above it.  With a near FP32's least normal number and
+    T = 1e-12 the quotient's residual a - q T is subnormal; the step must still take the rounded quotient,
+    as tv_tbar does.  The last row is 0, so after one step it is c tbar by the pair step: the product's two
+    parts added, the low one rounded to a subnormal number."""
+    n = 1500
+    og = O.Geometry(n, ny=2, V=4, U=8)
+    G = gpu_geometry(og)
+    rng = np.random.default_rng(4)
+    x = np.zeros((2, n), np.float32)
+    x[0, ::2] = rng.uniform(0.5e-37, 4e-37, n // 2)
+    x[0, 1::2] = 1e-12 * rng.uniform(0.5, 1.5, n // 2)
+    xd = to_dev(x)
+    _, nn, t = G.tv_tbar(xd)
+    gamma = 2e-13 * np.sqrt(nn)
+    rc, ell, trials = G.superiorize(xd, 0, 0.9, gamma, 1)
+    assert rc == 0 and trials == [1]
+    ct = float(np.float32(gamma / np.sqrt(nn))) * t.double().cpu().numpy()[1]     # exact in FP64
+    hi = ct.astype(np.float32)
+    want = hi + (ct - hi).astype(np.float32)
+    assert np.count_nonzero(want[::2]) > 700
+    np.testing.assert_array_equal(xd.cpu().numpy()[1], want)
