@@ -630,20 +630,28 @@ __device__ __noinline__ void stv_set_pow(StvScalars *s, double apow, double gamm
     s->gh = (float)s->gap;
     s->gl = (float)(s->gap - (double)s->gh);
 }
-// gamma a^l / sqrt(nn) rounded to FP32 (0 for nn = 0): on the FP32 pipe to about 2^-46 before the last
-// rounding, in FP64 outside its range.
+// gamma a^l / sqrt(nn) rounded to FP32 (0 for nn = 0): on the FP32 pipe, within 2^-44 before the last rounding;
+// in FP64, as k_stv has it, outside FP32's range and where an error of that size could turn the last rounding
+// (one step in 2^17).
 __device__ __noinline__ float stv_step(const StvScalars *s, double nn)
 {
     if (!(nn > 0.0)) return 0.0f;
     const float nh = (float)nn, gh = s->gh;
-    if (!(nh > 1e-30f && nh < 1e30f && gh > 1e-25f && gh < 1e25f)) return (float)(s->gap * rsqrt_fp64(nn));
-    const float nl = (float)(nn - (double)nh);
-    const float y = rsqrtf(nh);
-    const df m = df_mul(df{nh, nl}, df_prod(y, y));
-    const float e = __fsub_rn(__fsub_rn(1.0f, m.h), m.l);                          // 1 - nn y^2
-    const float yl = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, 0.5f * e));   // 1 / sqrt(nn) = y + yl
-    const df p = df_prod(gh, y);
-    return __fadd_rn(p.h, __fadd_rn(p.l, __fmaf_rn(gh, yl, __fmul_rn(s->gl, y))));
+    if (nh > 1e-30f && nh < 1e30f && gh > 1e-25f && gh < 1e25f) {
+        const float nl = (float)(nn - (double)nh);
+        const float y = rsqrtf(nh);
+        const df m = df_mul(df{nh, nl}, df_prod(y, y));
+        const float e = __fsub_rn(__fsub_rn(1.0f, m.h), m.l);                          // 1 - nn y^2
+        const float yl = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, 0.5f * e));   // 1 / sqrt(nn) = y + yl
+        const df p = df_prod(gh, y);
+        const float tail = __fadd_rn(p.l, __fmaf_rn(gh, yl, __fmul_rn(s->gl, y)));
+        const float c = __fadd_rn(p.h, tail);
+        // What c leaves of the sum, exactly: were it 2^-17 of itself more, would c be the same?  (Half a unit of c
+        // is 2^-25 c or more, and 2^-17 of it four times the error.)
+        const float rest = __fadd_rn(__fsub_rn(p.h, c), tail);
+        if (p.h > 1e-20f && p.h < 1e30f && __fadd_rn(c, __fmul_rn(rest, 1.0f + 0x1p-17f)) == c) return c;
+    }
+    return (float)(s->gap * rsqrt_fp64(nn));
 }
 __device__ __noinline__ void stv_first_pow(StvScalars *s, const Scal *sc, double a, double gamma)
 {

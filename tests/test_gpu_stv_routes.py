@@ -58,3 +58,31 @@ def test_one_step_on_an_image_whose_quotients_underflow():
     want = hi + (ct - hi).astype(np.float32)
     assert np.count_nonzero(want[::2]) > 700
     np.testing.assert_array_equal(xd.cpu().numpy()[1], want)
+
+
+@pytest.mark.parametrize("nx", [4, 6, 12, 38, 107])
+def test_step_length_is_rounded_from_fp64(nx):
+    """Two rows of 1 and 0: tbar is -1 above and 1 below but for the last column, so ||tbar||^2 = 2 (nx - 1)
+    exactly and the lower row is the step length c = RN(gamma / ||tbar||) itself.  gamma is taken so that
+    the exact quotient is 2^-49 beside the middle of two FP32 numbers, four times FP64's error (a rounded
+    reciprocal root and a product, 2^-51) and an eighth of a double-float product's."""
+    from decimal import Decimal, getcontext
+    getcontext().prec = 50
+    og = O.Geometry(nx, ny=2, V=4, U=8)
+    G = gpu_geometry(og)
+    root = Decimal(2 * (nx - 1)).sqrt()
+    rng = np.random.default_rng(nx)
+    for k in range(48):
+        lo = np.float32(rng.uniform(0.004, 0.016))
+        hi = np.nextafter(lo, np.float32(1))
+        mid = (Decimal(float(lo)) + Decimal(float(hi))) / 2
+        up = k % 2 == 0
+        gamma = float(mid * root * (1 + Decimal(2) ** -49 * (1 if up else -1)))
+        off = Decimal(gamma) / root / mid - 1
+        assert Decimal(2) ** -50 < abs(off) < Decimal(2) ** -48 and (off > 0) == up
+        xd = to_dev(np.stack([np.ones(nx), np.zeros(nx)]))
+        rc, ell, trials = G.superiorize(xd, 0, 0.9, gamma, 1)
+        assert rc == 0 and trials == [1]
+        want = np.full(nx, hi if up else lo)
+        want[-1] = 0.0
+        np.testing.assert_array_equal(xd.cpu().numpy()[1], want)
