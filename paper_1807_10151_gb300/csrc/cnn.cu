@@ -624,8 +624,8 @@ static int launch_wgrad(const __nv_bfloat16 *in, const __nv_bfloat16 *G, int cin
 // out[co][ci][dy][dx], then db: element e of the partials' order [dx][co][dy][ci] is
 // sum_b partial[b][e] in a fixed order: warp w of a block adds the partials b = w, w + 8, ...
 // for 32 consecutive e (lane = e), then warp 0 adds the eight warp sums in warp order.  Eight
-// loads in flight and double-float sums (about 48 bits, on the FP32 pipe): with FP64 adds, one
-// load at a time and a launch per layer the five layers took 65 us (32 x 128^2), 11 us now.
+// loads in flight and sums in three FP32 parts (no less accurate than FP64 ones, on the FP32 pipe): with
+// FP64 adds, one load at a time and a launch per layer the five layers took 65 us (32 x 128^2), 11 us now.
 struct ReduceArgs {
     const float *partial[kCnnLayers];
     float *out[kCnnLayers];
@@ -634,14 +634,14 @@ struct ReduceArgs {
 
 __global__ void __launch_bounds__(256) k_reduce(ReduceArgs a)
 {
-    __shared__ float2 sh[8][33];
+    __shared__ float sh[3][8][32];
     int l = kCnnLayers - 1;
     while (l > 0 && (int)blockIdx.x < a.first[l]) --l;
     const float *partial = a.partial[l];
     const int nb = a.nb[l], cout = a.cout[l], cin = a.cin[l];
     const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
     const int e = (blockIdx.x - a.first[l]) * 32 + ln, len = cout * cin * 9 + cout;
-    df s = df_make(0.0f);
+    tf s = tf_make();
     if (e < len) {
         int b = w;
         for (; b + 56 < nb; b += 64) {
@@ -649,27 +649,30 @@ __global__ void __launch_bounds__(256) k_reduce(ReduceArgs a)
 #pragma unroll
             for (int k = 0; k < 8; ++k) v[k] = partial[(size_t)(b + 8 * k) * len + e];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) df_acc(s, v[k]);
+            for (int k = 0; k < 8; ++k) tf_acc(s, v[k]);
         }
-        for (; b < nb; b += 8) df_acc(s, partial[(size_t)b * len + e]);
+        for (; b < nb; b += 8) tf_acc(s, partial[(size_t)b * len + e]);
     }
-    sh[w][ln] = make_float2(s.h, s.l);
+    sh[0][w][ln] = s.h;
+    sh[1][w][ln] = s.l;
+    sh[2][w][ln] = s.m;
     __syncthreads();
     if (w == 0 && e < len) {
-        df tot = df_make(0.0f);
+        tf sum = tf_make();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) tot = df_add(tot, df{sh[k][ln].x, sh[k][ln].y});
-        if (!isfinite(tot.h)) {   // an infinite partial (double-float sums turn it into NaN): the plain sum
+        for (int k = 0; k < 8; ++k) tf_add(sum, sh[0][k][ln], sh[1][k][ln], sh[2][k][ln]);
+        float tot = (float)tf_to_double(sum);
+        if (!isfinite(tot)) {   // an infinite partial (its TwoSum error is NaN): the plain sum
             double v = 0.0;
             for (int b = 0; b < nb; ++b) v += (double)partial[(size_t)b * len + e];
-            tot.h = (float)v;
+            tot = (float)v;
         }
         int o = e;
         if (e < 9 * cout * cin) {
             const int r = e / cin, ci = e - r * cin, dy = r % 3, co = (r / 3) % cout, dx = r / (3 * cout);
             o = (co * cin + ci) * 9 + dy * 3 + dx;
         }
-        a.out[l][o] = tot.h;
+        a.out[l][o] = tot;
     }
 }
 
@@ -677,7 +680,7 @@ __global__ void __launch_bounds__(256) k_reduce(ReduceArgs a)
 // Per-image unit-RMS scale factors sqrt(n / sum v^2) of x, tbar and (tg not null) the target
 // (0 for an all-zero image): scale[3 img + k].  Grid (nblk, count, arrays), nblk =
 // norm_blocks(n) <= kNormBlocks: each block sums a contiguous part of one image (exact
-// products, double-float sums: with FP64 products the narrow pipe held this at 31 us for
+// products, sums in three FP32 parts: with FP64 ones the narrow pipe held this at 31 us for
 // 8 x 512^2, 20 us now); the image's last block adds the partials in a fixed order and
 // writes the FP32 factor.
 constexpr int kNormBlocks = 256;
@@ -685,19 +688,33 @@ constexpr int kNormUnroll = 8;   // elements per thread in flight
 
 // s += v^2: exactly where v^2 and its rounding error are FP32 numbers, else into the FP64 sum
 // `rest` (*any then); their total over the block, in thread 0
-__device__ __forceinline__ void sq_acc(df &s, double &rest, bool &any, float v)
+__device__ __forceinline__ void sq_acc(tf &s, double &rest, bool &any, float v)
 {
     const float a = fabsf(v);
     if (v == 0.0f || (a > 1e-15f && a < 1e15f)) {
-        df_acc_prod(s, v, v);
+        tf_acc_sq(s, v);
     } else {
         rest += (double)v * (double)v;
         any = true;
     }
 }
-__device__ __forceinline__ double sq_total(df s, double rest, bool any, double *red)
+__device__ __forceinline__ double sq_total(tf s, double rest, bool any, double *red)
 {
-    const double v = block_sum_df<256>(s, red);
+    tf_warp_sum(s);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    float *f = reinterpret_cast<float *>(red);   // [8 warps][3]
+    if (l == 0) {
+        f[3 * w] = s.h;
+        f[3 * w + 1] = s.l;
+        f[3 * w + 2] = s.m;
+    }
+    __syncthreads();
+    double v = 0.0;
+    if (w == 0) {
+        s = l < 8 ? tf{f[3 * l], f[3 * l + 1], f[3 * l + 2]} : tf_make();
+        tf_warp_sum(s);
+        if (l == 0) v = tf_to_double(s);
+    }
     return __syncthreads_or(any) ? v + block_sum<256>(rest, red) : v;
 }
 
@@ -712,7 +729,7 @@ __global__ void __launch_bounds__(256) k_norms(const float *x, const float *tb, 
     const long long per = (n + nblk - 1) / nblk;
     const long long e0 = blk * per, e1 = e0 + per < n ? e0 + per : n;
     const float *vi = (which == 0 ? x : (which == 1 ? tb : tg)) + blockIdx.y * n;
-    df s = df_make(0.0f);
+    tf s = tf_make();
     double rest = 0.0;
     bool any = false;
     for (long long e = e0 + threadIdx.x; e < e1; e += 256 * kNormUnroll) {
@@ -763,7 +780,7 @@ __global__ void __launch_bounds__(256) k_loss(const float *out, const float *tar
                                               double *loss)
 {
     __shared__ __align__(16) double red[40];
-    df s = df_make(0.0f);
+    tf s = tf_make();
     double rest = 0.0;
     bool any = false;
     const float scale = (float)(2.0 / (double)total);

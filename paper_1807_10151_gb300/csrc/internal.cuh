@@ -370,6 +370,53 @@ __device__ __forceinline__ void df_acc(df &s, float v) { s = df_add(s, df{v, 0.0
 __device__ __forceinline__ void df_acc_prod(df &s, float a, float b) { s = df_add(s, df_prod(a, b)); }
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.h + (double)a.l; }
 
+// Sums that replace FP64 ones and must not be less accurate: three FP32 parts, the exact errors of the first
+// part's additions collected in the second and those of the second's in the third, so that only the third is
+// rounded (2^-24 of a part that is itself about 2^-48 of the sum).  On the FP32 pipe, 13 instructions per term.
+struct tf {
+    float h, l, m;
+};
+
+__device__ __forceinline__ float two_sum(float a, float b, float &e)   // a + b = result + e, exactly
+{
+    const float s = __fadd_rn(a, b), bv = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
+    return s;
+}
+__device__ __forceinline__ tf tf_make() { return {0.0f, 0.0f, 0.0f}; }
+__device__ __forceinline__ void tf_low(tf &s, float v)   // a term of the size of the second part
+{
+    float e;
+    s.l = two_sum(s.l, v, e);
+    s.m = __fadd_rn(s.m, e);
+}
+__device__ __forceinline__ void tf_acc(tf &s, float v)
+{
+    float e;
+    s.h = two_sum(s.h, v, e);
+    tf_low(s, e);
+}
+__device__ __forceinline__ void tf_acc_sq(tf &s, float v)   // v^2, exactly
+{
+    const df p = df_prod(v, v);
+    tf_acc(s, p.h);
+    tf_low(s, p.l);
+}
+__device__ __forceinline__ void tf_add(tf &s, float h, float l, float m)
+{
+    tf_acc(s, h);
+    tf_low(s, l);
+    s.m = __fadd_rn(s.m, m);
+}
+__device__ __forceinline__ void tf_warp_sum(tf &s)   // in lane 0, in a fixed order
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        tf_add(s, __shfl_down_sync(0xffffffffu, s.h, o), __shfl_down_sync(0xffffffffu, s.l, o),
+               __shfl_down_sync(0xffffffffu, s.m, o));
+}
+__device__ __forceinline__ double tf_to_double(const tf &s) { return (double)s.h + ((double)s.l + (double)s.m); }
+
 // ----------------------------------------------------------------- reductions
 __device__ __forceinline__ double warp_sum(double v)
 {
