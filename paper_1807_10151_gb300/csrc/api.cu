@@ -113,7 +113,7 @@ struct Workspace {
     int bwp = 0;                // widest window there
     int mirror = 0;             // 1: some problem has mirror pairs of views
     int stv_ti = 0;             // rows of k_stv_tile's tiles; 0: the images do not fit, S_TV walks them in memory
-    bool wc_ready = false;      // the problems' frequency tables are filled
+    bool wc_ready = false;      // the frequency tables are filled
     std::vector<void *> allocs;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t body_exec = nullptr;
@@ -610,6 +610,12 @@ extern "C" int supcg_destroy_geometry(supcg_geometry g)
 }
 
 // ------------------------------------------------------------------ workspace
+// The first problem with problem c's geometry.
+static int first_of(const std::vector<supcg_geometry> &gs, int c)
+{
+    return (int)(std::find(gs.begin(), gs.begin() + c, gs[c]) - gs.begin());
+}
+
 static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
 {
     auto *w = new (std::nothrow) Workspace();
@@ -724,6 +730,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         Prob &P = w->hp[c];
         const size_t img = (size_t)g->ny * g->nxp, imgT = (size_t)g->nx * g->nyp, sino = (size_t)g->V * g->Up;
         const size_t mir = g->npairs > 0 ? 1 : 0;   // mirrored images only with mirror pairs
+        const int same = first_of(gs, c);           // the first problem of this geometry holds its frequency table
         int maxblk = 0;
         for (int kt = 0; kt < KT_COUNT; ++kt) maxblk = std::max(maxblk, nb[kt][c]);
         const size_t npart = std::max<size_t>(std::max(12 * (size_t)nb[KT_STV][c], 4 * (size_t)nb[KT_STVT][c]), 2 * (size_t)maxblk) + 64;
@@ -735,7 +742,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
                                 (size_t)std::max(nb[KT_BWD][c], nb[KT_BWDP][c]) * 4, img * 4, img * 4,
                                 mir * img * 4, mir * imgT * 4, mir * img * 4, mir * imgT * 4,
                                 img * 4, imgT * 4, mir * img * 4, mir * imgT * 4, sino * 8, sino * 8,
-                                (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 16};
+                                same < c ? 0 : (size_t)(g->ny / 2 + 1) * (g->nx / 2 + 1) * 16};
         constexpr int kPieces = sizeof(sizes) / sizeof(sizes[0]);
         size_t total = 0;
         for (size_t s : sizes) total += al(s);
@@ -765,7 +772,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         P.dmT = mir ? (float *)ptrs[28] : nullptr;
         P.rd = (double *)ptrs[29];
         P.qd = (double *)ptrs[30];
-        P.wc = (double2 *)ptrs[31];
+        P.wc = same < c ? w->hp[same].wc : (double2 *)ptrs[31];
         if (mir) w->mirror = 1;
         P.border = g->dborder;
         P.border_all = g->dborder_all;
@@ -909,12 +916,17 @@ static int ops_ws(supcg_geometry g, int batch, Workspace **out)
     return SUPCG_OK;
 }
 
-// The preconditioner's filter: the workspace's table of frequencies on its first use, then D from mu and rho.
+// The preconditioner's filter: the workspace's tables of frequencies on its first use (one per geometry; a table
+// allocated with the geometry, for all its workspaces, made the first call at 512^2 40 us longer), then D from mu
+// and rho.
 static int enqueue_filter(Workspace *w, cudaStream_t st)
 {
     if (!w->wc_ready) {
-        const int rc = launch_fft_wc(w->L(KT_VEC, st));
-        if (rc) return rc;
+        for (int c = 0; c < w->count; ++c) {
+            if (first_of(w->geoms, c) < c) continue;
+            const int rc = launch_fft_wc(w->hp[c].wc, w->geoms[c]->nx, w->geoms[c]->ny, st);
+            if (rc) return rc;
+        }
         w->wc_ready = true;
     }
     return launch_fft_dtab(w->L(KT_VEC, st));

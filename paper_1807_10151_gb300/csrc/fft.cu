@@ -389,26 +389,23 @@ __global__ void __launch_bounds__(256) k_fft_cols(const Prob *__restrict__ probs
 
 // (w_r, cos w_r) on the quarter spectrum, w_i = 2 pi m_i / N_i, w_r = min(sqrt(w1^2 + w2^2), pi): kept with the
 // workspace, since the FP64 square root and cosine of every entry took 22 us per call on the narrow FP64 pipe.
-// Launched on the vector kernels' grid (about one entry per thread).
-__global__ void __launch_bounds__(256) k_fft_wc(const Prob *__restrict__ probs, const int *__restrict__ prefix, int count)
+__global__ void __launch_bounds__(256) k_fft_wc(double2 *__restrict__ wc, int nx, int ny)
 {
-    int local;
-    const int pi = find_problem(prefix, count, blockIdx.x, &local);
-    const Prob &P = probs[pi];
-    const int nx = P.nx, ny = P.ny, hx = nx / 2 + 1, hy = ny / 2 + 1, nblk = prefix[pi + 1] - prefix[pi];
+    const int hx = nx / 2 + 1, hy = ny / 2 + 1;
     const double two_pi = 6.28318530717958647692;
     const double pi_d = 3.14159265358979323846;
-    for (long long e = (long long)local * 256 + threadIdx.x; e < (long long)hx * hy; e += (long long)nblk * 256) {
+    for (long long e = (long long)blockIdx.x * 256 + threadIdx.x; e < (long long)hx * hy; e += (long long)gridDim.x * 256) {
         const int m1 = (int)(e / hx), m2 = (int)(e - (long long)m1 * hx);
         const double w1 = two_pi * m1 / ny, w2 = two_pi * m2 / nx;
         const double wr = fmin(sqrt(w1 * w1 + w2 * w2), pi_d);
-        P.wc[e] = make_double2(wr, cos(wr));
+        wc[e] = make_double2(wr, cos(wr));
     }
 }
 
-int launch_fft_wc(const Launch &L)
+int launch_fft_wc(double2 *wc, int nx, int ny, cudaStream_t st)
 {
-    k_fft_wc<<<L.blocks, 256, 0, L.st>>>(L.probs, L.prefix, L.count);
+    const long long n = (long long)(nx / 2 + 1) * (ny / 2 + 1);
+    k_fft_wc<<<(unsigned)std::min<long long>((n + 255) / 256, 1 << 16), 256, 0, st>>>(wc, nx, ny);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;
 }

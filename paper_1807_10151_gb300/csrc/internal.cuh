@@ -261,7 +261,7 @@ struct Prob {
     float *r, *q, *bpad;
     double *rd, *qd;
     double2 *C;            // FFT scratch [ny][nx] (FP64 complex)
-    double2 *wc;           // (w_r, cos w_r) on the quarter spectrum [ny/2+1][nx/2+1], for Dtab
+    double2 *wc;           // (w_r, cos w_r) on the quarter spectrum [ny/2+1][nx/2+1], for Dtab; one per geometry
     float2 *Dtab;          // h(w_r) / (nx ny) at (min(k1, ny-k1), min(k2, nx-k2)), double-float: [ny/2+1][nx/2+1]
     float2 *bsplit;        // backprojector: each sinogram's and view part's pixel sums, double-float [2][bparts][ny][nxp]
     int bparts;            // backprojector: blocks per pixel tile, each taking a contiguous share of the view chunks
@@ -807,7 +807,7 @@ int launch_stage_sino(const Launch &L);                     // caller sinogram i
 int launch_store_out(const Launch &L, int which, const Io &io = Io());   // padded image (0 x, 1 tbar, 2 g) -> caller
 int launch_fft_rows(const Launch &L, int inverse, int standalone, int smem, const Io &io = Io());
 int launch_fft_cols(const Launch &L, int standalone, int smem);
-int launch_fft_wc(const Launch &L);                         // fills wc (once per workspace)
+int launch_fft_wc(double2 *wc, int nx, int ny, cudaStream_t st);   // fills wc (once per workspace)
 int launch_fft_dtab(const Launch &L);                       // fills Dtab from mu, rho (once per solve or call)
 int launch_gray(const Launch &L);                           // sc->muX from bpad (Bayesian criterion)
 int launch_pupdate(const Launch &L);
