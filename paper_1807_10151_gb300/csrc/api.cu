@@ -624,12 +624,12 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
     w->geoms = gs;
     for (const supcg_geometry g : gs) w->versions.push_back(g->layout_version);
     w->hp.resize(w->count);
-    int dev = 0, nsm = 0, per_sm = 0;
+    int dev = 0, nsm = 0, stv_cap = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int rc = stv_max_blocks_per_sm(&per_sm);
+    int rc = stv_max_blocks(&stv_cap);
     if (rc) { delete w; return rc; }
-    const int stv_cap = std::max(1, nsm * per_sm);
+    stv_cap = std::max(1, stv_cap);
     if (w->count > stv_cap) { delete w; return SUPCG_ERR_UNSUPPORTED; }
 
     // blocks per problem for every kernel type
@@ -712,13 +712,14 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
         hprefix[kt * (w->count + 1) + w->count] = acc;
         w->blocks[kt] = acc;
     }
-    // the prefix tables, then the problems' scalars and the inline trial counts
+    // the prefix tables, then (zeros, in the same copy) the problems' scalars and the inline trial counts
     const size_t prefix_bytes = (sizeof(int) * hprefix.size() + 255) / 256 * 256;
     const size_t scal_bytes = sizeof(Scal) * w->count + kInlineTrials * sizeof(int);
+    static_assert(sizeof(Scal) % sizeof(int) == 0, "a whole number of table entries");
+    hprefix.resize((prefix_bytes + scal_bytes) / sizeof(int), 0);
     if (cudaMalloc(&w->dprefix, prefix_bytes + scal_bytes) != cudaSuccess) { delete w; return SUPCG_ERR_NOMEM; }
     w->scals = reinterpret_cast<Scal *>(reinterpret_cast<char *>(w->dprefix) + prefix_bytes);
-    if (cudaMemset(w->scals, 0, scal_bytes) != cudaSuccess ||
-        cudaEventCreateWithFlags(&w->last, cudaEventDisableTiming) != cudaSuccess ||
+    if (cudaEventCreateWithFlags(&w->last, cudaEventDisableTiming) != cudaSuccess ||
         cudaMemcpy(w->dprefix, hprefix.data(), sizeof(int) * hprefix.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         delete w;
         return SUPCG_ERR_CUDA;
@@ -832,6 +833,31 @@ int supcg::func_attrs_once(const void *func, int max_dyn_smem, int carveout)
     SUPCG_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_smem));
     if (carveout >= 0) SUPCG_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, carveout));
     done.emplace_back(func, dev);
+    return SUPCG_OK;
+}
+
+int supcg::resident_blocks(const void *func, int threads, size_t smem, int *out)
+{
+    struct Known {
+        const void *func;
+        int dev, blocks;
+    };
+    static std::mutex mu;
+    static std::vector<Known> known;
+    int dev = 0;
+    int rc = current_device(&dev);
+    if (rc) return rc;
+    std::lock_guard<std::mutex> lk(mu);
+    for (const Known &k : known)
+        if (k.func == func && k.dev == dev) {
+            *out = k.blocks;
+            return SUPCG_OK;
+        }
+    int nsm = 0, per_sm = 0;
+    SUPCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, func, threads, smem));
+    *out = nsm * per_sm;
+    known.push_back({func, dev, *out});
     return SUPCG_OK;
 }
 

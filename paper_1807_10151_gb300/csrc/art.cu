@@ -255,15 +255,7 @@ static int with_art_rows(int side, F &&f)
 
 int art_max_blocks(int side, int *out)
 {
-    int nsm = 0, per_sm = 0, dev = 0;
-    SUPCG_CUDA_TRY(cudaGetDevice(&dev));
-    SUPCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int rc = with_art_rows(side, [&](auto *kernel) -> int {
-        SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kArtRayThreads, 0));
-        return SUPCG_OK;
-    });
-    *out = nsm * per_sm;
-    return rc;
+    return with_art_rows(side, [&](auto *kernel) { return resident_blocks((const void *)kernel, kArtRayThreads, 0, out); });
 }
 
 int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st)

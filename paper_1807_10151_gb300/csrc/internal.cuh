@@ -766,6 +766,9 @@ int cuda_fail(cudaError_t e, const char *what, const char *file, int line);
 // kernel's dynamic shared-memory limit to max_dyn_smem bytes and, when carveout >= 0,
 // set its preferred shared-memory carveout.  Thread-safe.
 int func_attrs_once(const void *func, int max_dyn_smem, int carveout = -1);
+// Blocks of a kernel that fit the current device at once (with its attributes set), asked of the driver once per
+// (kernel, device): a kernel has one block size and one shared-memory size here.  Thread-safe.
+int resident_blocks(const void *func, int threads, size_t smem, int *out);
 // Current device (0 .. kMaxDevices-1) for per-device host caches.
 constexpr int kMaxDevices = 64;
 int current_device(int *dev);
@@ -818,7 +821,7 @@ int launch_gather_xt(const Launch &L, float *xs, float *ts);   // x, tbar of eve
 int launch_stv(const Launch &L, int K, double a, double gamma, long long max_trials, int *trials_out,
                int want_snorm, const float *dir = nullptr);
 int launch_tv_tbar(const Launch &L);
-int stv_max_blocks_per_sm(int *out);
+int stv_max_blocks(int *out);                   // co-resident blocks of k_stv
 int stv_tiles(int nx, int ny, int ti);          // blocks of k_stv_tile for an image, tiles of ti x 32 pixels
 int stv_tile_max_blocks(int ti, int *out);      // co-resident blocks of k_stv_tile
 int launch_stv_tile(const Launch &L, int ti, int K, double a, double gamma, long long max_trials, int *trials_out,

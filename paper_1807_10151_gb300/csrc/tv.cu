@@ -943,12 +943,7 @@ static int stv_tile_blocks_t(int *out)
 {
     int rc = func_attrs_once((const void *)k_stv_tile<TI>, (int)sizeof(StvTile<TI>), (int)cudaSharedmemCarveoutMaxShared);
     if (rc) return rc;
-    int dev = 0, nsm = 0, per_sm = 0;
-    SUPCG_CUDA_TRY(cudaGetDevice(&dev));
-    SUPCG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stv_tile<TI>, kStvThreads, sizeof(StvTile<TI>)));
-    *out = nsm * per_sm;
-    return SUPCG_OK;
+    return resident_blocks((const void *)k_stv_tile<TI>, kStvThreads, sizeof(StvTile<TI>), out);
 }
 int stv_tile_max_blocks(int ti, int *out)
 {
@@ -981,11 +976,7 @@ int launch_stv_tile(const Launch &L, int ti, int K, double a, double gamma, long
     return launch_stv_tile_t<128>(L, K, a, gamma, max_trials, trials_out, want_snorm);
 }
 
-int stv_max_blocks_per_sm(int *out)
-{
-    SUPCG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_stv, kTvThreads, 0));
-    return SUPCG_OK;
-}
+int stv_max_blocks(int *out) { return resident_blocks((const void *)k_stv, kTvThreads, 0, out); }
 
 int launch_stv(const Launch &L, int K, double a, double gamma, long long max_trials, int *trials_out,
                int want_snorm, const float *dir)
