@@ -96,7 +96,7 @@ enum { KT_FWD, KT_FWDA, KT_BWD, KT_BWDP, KT_VEC, KT_TR, KT_ROWS, KT_COLS, KT_SIN
 struct Workspace {
     int count = 0;
     std::vector<supcg_geometry> geoms;
-    std::vector<unsigned> versions;   // the geometries' layout versions when this was built
+    std::vector<unsigned long long> versions;   // the geometries' layout versions when this was built
     std::vector<Prob> hp;
     std::vector<Prob> on_device;      // what dp holds (empty: nothing yet)
     Prob *dp = nullptr;
@@ -155,6 +155,12 @@ struct Workspace {
     }
 };
 
+static unsigned long long new_layout_version()
+{
+    static std::atomic<unsigned long long> last{0};
+    return ++last;
+}
+
 struct supcg_geometry_s {
     int nx, ny, V, U, storage;
     double d, ds, off;
@@ -192,7 +198,9 @@ struct supcg_geometry_s {
     Workspace *ws_batch = nullptr;  // batched solve owned by this (first) geometry
     std::vector<supcg_geometry> batch_key;
     int bparts = kBwdViewParts;     // backprojector: view parts per pixel tile
-    unsigned layout_version = 0;    // changed with the tiling: workspaces built before are stale
+    // changed with the tiling: workspaces built before are stale.  No two geometries ever have the same one, so that
+    // a batch's workspace does not take a new geometry for a destroyed one whose address it got.
+    unsigned long long layout_version = new_layout_version();
 };
 
 // Forward projector box width: the inner indices that one warp's 64 rays can
@@ -548,7 +556,7 @@ extern "C" int supcg_set_tiling(supcg_geometry g, int fwd_bins_per_block)
     free_ws(g->ws_solve);
     free_ws(g->ws_batch);
     g->ops_batch = 0;
-    ++g->layout_version;
+    g->layout_version = new_layout_version();
     return SUPCG_OK;
 }
 
@@ -561,7 +569,7 @@ extern "C" int supcg_set_bwd_parts(supcg_geometry g, int parts)
     free_ws(g->ws_solve);
     free_ws(g->ws_batch);
     g->ops_batch = 0;
-    ++g->layout_version;
+    g->layout_version = new_layout_version();
     return SUPCG_OK;
 }
 
