@@ -118,7 +118,7 @@ struct Workspace {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t body_exec = nullptr;
     double key[6] = {};         // parameters the captured body depends on
-    int key_i[4] = {};
+    unsigned long long key_i[3] = {};
     int *trials_dev = nullptr;
     int trials_cap = 0;
     long long body_nodes = 0;
@@ -1364,7 +1364,10 @@ static int run_solve(Workspace *w, const float *const *d_b, float *const *d_x, c
     if (use_graph) {
         const double key[6] = {p->a, p->gamma, (double)p->max_trials, (double)p->K, (double)p->perturb,
                                (double)p->precondition};
-        const int key_i[4] = {want_snorm, 1, (int)((uintptr_t)d_trace & 0x7fffffff), (int)((uintptr_t)net & 0x7fffffff)};
+        // (the network by its number: the body holds its buffers' addresses, and a new network may get a destroyed
+        // one's address with buffers elsewhere)
+        const unsigned long long key_i[3] = {(unsigned long long)want_snorm, (unsigned long long)(uintptr_t)d_trace,
+                                             net ? cnn_id(net) : 0};
         if (!w->body_exec || memcmp(key, w->key, sizeof(key)) || memcmp(key_i, w->key_i, sizeof(key_i))) {
             if (w->body_exec) cudaGraphExecDestroy(w->body_exec);
             w->body_exec = nullptr;

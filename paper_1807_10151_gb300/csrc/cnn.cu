@@ -34,6 +34,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -859,7 +860,14 @@ __global__ void k_pack_weights(const float *W, int cout, int cin, int cin_real, 
 // ------------------------------------------------------------------ network object
 using namespace supcg;
 
+static unsigned long long next_cnn_id()
+{
+    static std::atomic<unsigned long long> last{0};
+    return ++last;
+}
+
 struct supcg_cnn_s {
+    const unsigned long long id = next_cnn_id();
     int ny, nx, cap;             // image size and the largest batch the buffers hold
     int nparam;
     int off_w[kCnnLayers], off_b[kCnnLayers];
@@ -1111,6 +1119,7 @@ int cnn_forward(supcg_cnn net, const float *d_x, const float *d_tbar, int count,
 
 namespace supcg {
 float *cnn_output(supcg_cnn net) { return net->out; }
+unsigned long long cnn_id(supcg_cnn net) { return net->id; }
 int cnn_shape(supcg_cnn net, int *ny, int *nx)
 {
     *ny = net->ny;

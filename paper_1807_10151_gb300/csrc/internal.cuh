@@ -828,6 +828,7 @@ int launch_stv_tile(const Launch &L, int ti, int K, double a, double gamma, long
                     int want_snorm);
 int cnn_forward(struct supcg_cnn_s *net, const float *d_x, const float *d_tbar, int count, cudaStream_t st);
 float *cnn_output(struct supcg_cnn_s *net);
+unsigned long long cnn_id(struct supcg_cnn_s *net);   // > 0, and no other network's, destroyed ones' included
 int cnn_shape(struct supcg_cnn_s *net, int *ny, int *nx);
 int cnn_capacity(struct supcg_cnn_s *net, int *max_batch);
 
