@@ -297,7 +297,8 @@ int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const supcg_art_pa
  * activations, FP32 accumulation (tensor cores), FP32 master weights (Adam).
  * Parameters, as a flat FP32 array: for each layer W[cout][cin][3][3] then
  * b[cout].  A network is created for images of ny x nx and up to max_batch
- * images per call; it owns its device memory.
+ * images per call; it owns its device memory: per image 448 bytes for each of
+ * (ny + 2) x (nx rounded up to 16, + 8) positions and 4 per pixel, and 35 MB.
  * ------------------------------------------------------------------------ */
 typedef struct supcg_cnn_s *supcg_cnn;
 

@@ -874,7 +874,9 @@ struct supcg_cnn_s {
     float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
     __nv_bfloat16 *wf[kCnnLayers] = {}, *wb[kCnnLayers] = {};
     __nv_bfloat16 *act[kCnnLayers] = {};   // act[0] input (16 ch), act[1..4] hidden (32 ch)
-    __nv_bfloat16 *gbuf[kCnnLayers] = {};  // gbuf[4] = dL/dout (16 ch); gbuf[l] = dL/dz_l (32 ch), l = 1..3; gbuf[0] for layer 1
+    // gbuf[4] = dL/dout (16 ch); gbuf[l] = dL/dz of layer l's output (32 ch), in two buffers by turns: the backward
+    // pass is done with gbuf[l] when gbuf[l - 2] is written
+    __nv_bfloat16 *gbuf[kCnnLayers] = {};
     float *out = nullptr, *partial[kCnnLayers] = {};   // partial: the layers' weight-gradient partials
     float *scales = nullptr;      // per image: factors of x, tbar and the target to unit RMS
     double *npart = nullptr, *lpart = nullptr;
@@ -956,7 +958,9 @@ extern "C" int supcg_cnn_create(int ny, int nx, int max_batch, unsigned long lon
         // one column after the last plane)
         const size_t cols = ((size_t)max_batch * (ny + 2) + 1) * act_pitch(nx);
         if (!rc) rc = cnn_alloc(net, (void **)&net->act[l], 2 * (cols * (l == 0 ? kInCh : kCh) + 64));
-        if (!rc) rc = cnn_alloc(net, (void **)&net->gbuf[l], 2 * (cols * (l == kCnnLayers - 1 ? kInCh : kCh) + 64));
+        const int last = l == kCnnLayers - 1;
+        if (!rc && (l < 2 || last)) rc = cnn_alloc(net, (void **)&net->gbuf[l], 2 * (cols * (last ? kInCh : kCh) + 64));
+        if (l >= 2 && !last) net->gbuf[l] = net->gbuf[l - 2];
     }
     int dev = 0, nsm = 1;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
