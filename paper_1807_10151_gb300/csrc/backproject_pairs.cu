@@ -163,7 +163,6 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward_pairs(co
 #pragma unroll
     for (int h = 0; h < NS * PX / 2; ++h) part2[h] = comp2[h] = pk2(0.0f, 0.0f);
 
-    const float *sino0 = (!DUAL && mode == BWD_H) ? P.q : P.r;
     const void *user = io.in + (size_t)pi * io.in_step;
     const int Up = P.Up;
     // tile corners in pixel-centre coordinates, of the left side
@@ -228,7 +227,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward_pairs(co
                         for (int k = 0; k < 2; ++k)
                             if (ub + k < P.U) y[a][k] = load_user(user, o + k, io.storage);
                     } else {
-                        const float *sn = (DUAL && (a & 1)) ? P.q : sino0;
+                        const float *sn = (DUAL && (a & 1)) ? P.q : P.r;
                         const float2 f = __ldg(reinterpret_cast<const float2 *>(sn + (size_t)v * Up + ub));
                         y[a][0] = f.x; y[a][1] = f.y;
                     }

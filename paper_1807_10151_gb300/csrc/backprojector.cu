@@ -100,8 +100,8 @@ __device__ __forceinline__ void bwd_view_x2(const ViewP &vp, float pb0, const ui
     }
 }
 
-// R^T y over one sinogram (mode BWD_G: y = r into g, BWD_H: y = q into h,
-// BWD_PLAIN: the caller's sinogram into the caller's image, or into g where io has none), or, DUAL, over two in one pass:
+// R^T y over one sinogram (mode BWD_G: y = r into g, BWD_PLAIN: the caller's sinogram
+// into the caller's image, or into g where io has none), or, DUAL, over two in one pass:
 // g from r and h from q (h = A p for the beta of the next step of Algorithm 2,
 // deferred to this pass: alpha takes p^T A p from the forward projector's ||q||^2).
 // FIXED_PARTS: the view parts per tile when every problem of the launch has that
@@ -155,8 +155,6 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
     for (int h = 0; h < PX / 2; ++h) Y2[h] = pk2(Y[2 * h], Y[2 * h + 1]);
     const uint64_t X2 = pk2(X, X);
 
-    const float *sino0 = (!DUAL && mode == BWD_H) ? P.q : P.r;
-    const float *sino1 = P.q;
     const void *user = io.in + (size_t)pi * io.in_step;
     const int Up = P.Up;
     // tile corners in pixel-centre coordinates
@@ -216,7 +214,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
                     if (ub + 2 < P.U) val.z = load_user(user, o + 2, io.storage);
                     if (ub + 3 < P.U) val.w = load_user(user, o + 3, io.storage);
                 } else {
-                    val = __ldg(reinterpret_cast<const float4 *>((s ? sino1 : sino0) + (size_t)v * Up + ub));
+                    val = __ldg(reinterpret_cast<const float4 *>((s ? P.q : P.r) + (size_t)v * Up + ub));
                 }
                 const float pl = vsh[buf][vv].P;   // the weights are in units of the view's plateau length
                 val.x = __fmul_rn(val.x, pl);

@@ -43,9 +43,7 @@ __device__ __forceinline__ void bwd_finish(const Prob &P, int ntiles, int pi, in
             }
     if (t == 0 && *bad_sh && P.sc) atomicExch(&P.sc->status, (int)SUPCG_ERR_UNSUPPORTED);
     if (!last_block(&P.tilecnt[tile], parts, last_sh)) return;
-    // output s: the gradient (g from r) or h from q
-    const bool is_g[2] = {DUAL || mode != BWD_H, false};
-    float *outs[2] = {(!DUAL && mode == BWD_H) ? P.h : P.g, P.h};
+    // output s: 0 the gradient (g from r), 1 h from q
     // Bayesian criterion (Eq. (2.3)): g = r^2 R^T r + (x - mu_X), h = r^2 R^T q + p, and
     // ||x - mu_X||^2 for f.  With a reference image, the selective error of Eq. (4.1) of
     // x = x_{k+1/2} over the centred ellipse S (this pass reads x anyway).
@@ -70,9 +68,10 @@ __device__ __forceinline__ void bwd_finish(const Prob &P, int ntiles, int pi, in
 #pragma unroll
                     for (int h = 0; h < kBwdMaxParts; ++h)
                         if (h < parts) vs = df_add(vs, df{pv[h].x, pv[h].y});
+                    float *out = s ? P.h : P.g;
                     if (bayes) {
                         double v = (double)vs.h + (double)vs.l;
-                        if (is_g[s]) {
+                        if (s == 0) {
                             const double dx = (double)P.x[o] - muX;
                             v = P.r2 * v + dx;
                             sx += dx * dx;
@@ -80,19 +79,19 @@ __device__ __forceinline__ void bwd_finish(const Prob &P, int ntiles, int pi, in
                             v = P.r2 * v + (double)P.p[o];
                         }
                         const float vh = (float)v;
-                        outs[s][o] = vh;
-                        if (solve && is_g[s]) P.glo[o] = (float)(v - (double)vh);
+                        out[o] = vh;
+                        if (solve && s == 0) P.glo[o] = (float)(v - (double)vh);
                     } else {
                         const float vh = __fadd_rn(vs.h, vs.l);   // the pair rounded to FP32
                         if (solve || !io.out) {
-                            outs[s][o] = vh;
+                            out[o] = vh;
                         } else {   // the caller's image
-                            void *out = io.out + (size_t)pi * io.out_step;
+                            void *user = io.out + (size_t)pi * io.out_step;
                             const size_t oc = (size_t)i * P.nx + j;
-                            if (io.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(out)[oc] = __float2bfloat16_rn(vh);
-                            else reinterpret_cast<float *>(out)[oc] = vh;
+                            if (io.storage == SUPCG_BF16) reinterpret_cast<__nv_bfloat16 *>(user)[oc] = __float2bfloat16_rn(vh);
+                            else reinterpret_cast<float *>(user)[oc] = vh;
                         }
-                        if (solve && is_g[s]) P.glo[o] = __fsub_rn(vs.l, __fsub_rn(vh, vs.h));   // its error, exactly
+                        if (solve && s == 0) P.glo[o] = __fsub_rn(vs.l, __fsub_rn(vh, vs.h));   // its error, exactly
                     }
                     if (want_se && s == 0) {   // pixel centre inside the ellipse (FP64, as the definition)
                         const double ex = ((double)j - 0.5 * (P.nx - 1)) / P.se_ax;
@@ -105,7 +104,7 @@ __device__ __forceinline__ void bwd_finish(const Prob &P, int ntiles, int pi, in
                 }
             }
     if (t == 0) P.tilecnt[tile] = 0;   // ready for the next launch
-    if (!(bayes && is_g[0]) && !want_se) return;
+    if (!bayes && !want_se) return;
     // the tiles' sums, added in tile order by the last tile to finish: f = r^2 ||R x - b||^2 +
     // ||x - mu_X||^2, and SE = sqrt(sum over S)
     const double bs = block_sum<kBwdThreads>(sx, red);

@@ -778,7 +778,8 @@ int current_device(int *dev);
 // FWD_RESID: r = R x - b (steps 1-9); FWD_NORM: q = R p and alpha; FWD_PLAIN: the caller's
 // projection; FWD_RUPD: r <- r + alpha q + R d (a while-body with S_TV)
 enum FwdMode { FWD_RESID = 0, FWD_NORM = 1, FWD_PLAIN = 2, FWD_RUPD = 3 };
-enum BwdMode { BWD_G = 0, BWD_H = 1, BWD_PLAIN = 2 };
+// BWD_G: the solver's gradient (and, in the dual pass, h); BWD_PLAIN: the caller's backprojection
+enum BwdMode { BWD_G = 0, BWD_PLAIN = 1 };
 
 struct Launch {
     const Prob *probs;     // device
