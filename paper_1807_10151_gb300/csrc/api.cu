@@ -1201,8 +1201,7 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_init(w->L(KT_VEC, st), s0));
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_stage_sino(w->L(KT_SINO, st)));      // b -> bpad
     if (isnan(p->mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
-    const int init_blocks = (int)std::min<size_t>(8192, (m + 63) / 64);
-    LAUNCH(SUPCG_KIND_VECTOR, st, launch_art_init(w->dp, p->r, init_blocks, st));   // norms, u = 0, x = mu_X
+    LAUNCH(SUPCG_KIND_VECTOR, st, launch_art_init(w->dp, p->r, (long long)m, st));   // norms, u = 0, x = mu_X
     int cap = 0;
     const int side = std::max(g->nx, g->ny);
     if ((rc = art_max_blocks(side, &cap))) return rc;

@@ -16,11 +16,14 @@
 // the ray sum <R_i, x> (a Kahan-compensated FP32 sum per thread, the
 // threads' pairs added in double-float arithmetic) and again for the update
 // (FP32 FMA).  One block per ray: its threads take a few rows each.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace supcg {
 
-constexpr int kArtThreads = 64;      // k_art_init: one ray per thread
+constexpr int kArtThreads = 64;      // k_art_init
+constexpr int kArtLanes = 8;         // its lanes per ray
 constexpr int kArtRayThreads = 256;  // k_art: one block per ray of a class
 
 // The per-ray constants of a ray's entries (the projectors' exact split).
@@ -75,20 +78,27 @@ __device__ __forceinline__ void art_row(const Prob &P, const ViewP &vp, const Ar
 }
 
 // 1 / (1 + r^2 ||R_i||^2) for every ray (FP64), u = 0, and x = mu_X on the image
-// (the starting point of the method).  One ray per thread (no pixel is read, so neither
-// the rows' order nor their spread over lanes matters), its squares summed in double-float
-// arithmetic: with a warp per ray and FP64 squares the narrow FP64 pipe held this at
-// 2.35 ms for the 522000 rays of 512^2 / 720 views, 0.60 ms now.
+// (the starting point of the method).  Eight lanes per ray (no pixel is read, so the
+// rows' order does not matter), its exact squares summed in double-float arithmetic:
+// with a warp per ray and FP64 squares the narrow FP64 pipe held this at
+// 2.35 ms for the 522000 rays of 512^2 / 720 views, 0.45 ms now.  A call without
+// cycles, us, with a warp per ray (FP64), 1 lane, 4, 8 and 16: 64^2 / 40 views 84, 92, 78, 72,
+// 73; 512^2 / 90 393, 219, 157, 144, 153; 512^2 / 720 2565, 655, 625, 653, 691; 1500 x 64 / 40
+// 202, 383, 148, 122, 102 (one lane's rays are a serial chain of up to 1500 rows).
 __global__ void __launch_bounds__(kArtThreads) k_art_init(const Prob *__restrict__ probs, double r)
 {
     const Prob &P = probs[0];
     const long long rays = (long long)P.V * P.U;
-    for (long long i = (long long)blockIdx.x * kArtThreads + threadIdx.x; i < rays; i += (long long)gridDim.x * kArtThreads) {
-        const int v = (int)(i / P.U), u = (int)(i - (long long)v * P.U);
+    const int lane = threadIdx.x % kArtLanes;
+    constexpr int PER = kArtThreads / kArtLanes;   // rays per block and turn
+    for (long long b = (long long)blockIdx.x * PER; b < rays; b += (long long)gridDim.x * PER) {
+        const long long i = b + threadIdx.x / kArtLanes;
+        const bool have = i < rays;
+        const int v = have ? (int)(i / P.U) : 0, u = have ? (int)(i - (long long)v * P.U) : 0;
         const ViewP vp = P.views[v];
         const ArtRay R = art_ray_setup(P, vp, u);
         df s = df_make(0.0f);
-        for (int o = R.lo; o <= R.hi; ++o) {
+        for (int o = R.lo + lane; o <= R.hi; o += kArtLanes) {
             int pix[3];
             float w[3];
             art_row(P, vp, R, o, pix, w);
@@ -96,9 +106,14 @@ __global__ void __launch_bounds__(kArtThreads) k_art_init(const Prob *__restrict
             for (int k = 0; k < 3; ++k)
                 if (w[k] != 0.0f) df_acc_prod(s, w[k], w[k]);
         }
-        const double pl = (double)vp.P;
-        P.art_rn[i] = 1.0 / (1.0 + r * r * pl * pl * df_to_double(s));
-        P.art_u[i] = 0.0;
+#pragma unroll
+        for (int o = kArtLanes / 2; o > 0; o >>= 1)
+            s = df_add(s, df{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)});
+        if (have && lane == 0) {
+            const double pl = (double)vp.P;
+            P.art_rn[i] = 1.0 / (1.0 + r * r * pl * pl * df_to_double(s));
+            P.art_u[i] = 0.0;
+        }
     }
     const float mu = (float)P.sc->muX;
     const size_t n = (size_t)P.ny * P.nxp;
@@ -258,8 +273,9 @@ int art_max_blocks(int side, int *out)
     return with_art_rows(side, [&](auto *kernel) { return resident_blocks((const void *)kernel, kArtRayThreads, 0, out); });
 }
 
-int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st)
+int launch_art_init(const Prob *d_prob, double r, long long rays, cudaStream_t st)
 {
+    const int blocks = (int)std::min<long long>(8192, (rays * kArtLanes + kArtThreads - 1) / kArtThreads);
     k_art_init<<<blocks, kArtThreads, 0, st>>>(d_prob, r);
     SUPCG_CUDA_TRY(cudaGetLastError());
     return SUPCG_OK;

@@ -797,7 +797,7 @@ int launch_forward(const Launch &L, const Launch &La, int which, int mode, const
 int launch_backward(const Launch &L, int mode, int bwin, const Io &io = Io());   // BWD_PLAIN: caller sinogram -> caller image
 int launch_backward2(const Launch &L, int bwin);   // g from r and h from q in one pass
 int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side the longer one of the image
-int launch_art_init(const Prob *d_prob, double r, int blocks, cudaStream_t st);
+int launch_art_init(const Prob *d_prob, double r, long long rays, cudaStream_t st);
 int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
 int backward_blocks(int nx, int ny, int parts, int ti);
 int backward_pairs_blocks(int nx, int ny, int parts, int ti);
