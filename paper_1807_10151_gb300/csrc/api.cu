@@ -1203,17 +1203,16 @@ extern "C" int supcg_art(supcg_geometry g, const float *d_b, float *d_x, const s
     if (isnan(p->mu)) LAUNCH(SUPCG_KIND_VECTOR, st, launch_gray(w->L(KT_SINO, st)));
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_art_init(w->dp, p->r, (long long)m, st));   // norms, u = 0, x = mu_X
     int cap = 0;
-    const int side = std::max(g->nx, g->ny);
-    if ((rc = art_max_blocks(side, &cap))) return rc;
+    if ((rc = art_max_blocks(g->nx, g->ny, &cap))) return rc;
     const int rays = (g->U + g->art_S - 1) / g->art_S;   // rays per class, one block each
     const int blocks = std::max(1, std::min(cap, rays));
     if (p->K == 0) {
         if (p->cycles > 0)
-            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, side, p->cycles, p->r, p->lambda, g->art_S, blocks, st));
+            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, g->nx, g->ny, p->cycles, p->r, p->lambda, g->art_S, blocks, st));
     } else {
         for (int c = 0; c < p->cycles; ++c) {   // SupART: S_TV, then one cycle
             LAUNCH(SUPCG_KIND_STV, st, enqueue_stv(w, st, p->K, p->a, p->gamma, p->max_trials, nullptr, 0));
-            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, side, 1, p->r, p->lambda, g->art_S, blocks, st));
+            LAUNCH(SUPCG_KIND_FORWARD, st, launch_art(w->dp, g->nx, g->ny, 1, p->r, p->lambda, g->art_S, blocks, st));
         }
     }
     LAUNCH(SUPCG_KIND_VECTOR, st, launch_store_out(w->L(KT_VEC, st), 0, io));

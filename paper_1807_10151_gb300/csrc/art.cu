@@ -81,7 +81,7 @@ __device__ __forceinline__ void art_row(const Prob &P, const ViewP &vp, const Ar
 // (the starting point of the method).  Eight lanes per ray (no pixel is read, so the
 // rows' order does not matter), its exact squares summed in double-float arithmetic:
 // with a warp per ray and FP64 squares the narrow FP64 pipe held this at
-// 2.35 ms for the 522000 rays of 512^2 / 720 views, 0.45 ms now.  A call without
+// 2.35 ms for the 522000 rays of 512^2 / 720 views, 0.60 ms now.  A call without
 // cycles, us, with a warp per ray (FP64), 1 lane, 4, 8 and 16: 64^2 / 40 views 84, 92, 78, 72,
 // 73; 512^2 / 90 393, 219, 157, 144, 153; 512^2 / 720 2565, 655, 625, 653, 691; 1500 x 64 / 40
 // 202, 383, 148, 122, 102 (one lane's rays are a serial chain of up to 1500 rows).
@@ -259,18 +259,24 @@ __global__ void __launch_bounds__(kArtRayThreads) k_art(const Prob *__restrict__
     }
 }
 
-// Rows per thread: enough for the longest ray in one group, up to 4 (images up to 1024 rows and columns).
+// Rows per thread.  One or two where they hold the longest ray in one group; beyond 512 rows or columns 4 where most
+// rays are long (both sides above 512 and 1536 together), else 2 and further groups: four rows take 124 registers,
+// so the device holds 304 blocks instead of 456, and a block's further rays of a class are prepared one after the
+// other.  Two classes (a view), us, with 2 and 4 rows: 513^2 10.8 and 12.4, 700^2 14.4 and 15.6, 768^2 16.7 and
+// 16.6, 850^2 19.2 and 17.4, 900^2 20.8 and 22.0, 1024^2 25.8 and 22.1, 2048^2 114 and 96; 1100 x 300 14.4 and 18.0,
+// 1500 x 64 15.1 and 19.2, 2048 x 400 25.2 and 29.8, 1400 x 800 31.4 and 29.0, 2048 x 700 39.6 and 36.4.
 template <typename F>
-static int with_art_rows(int side, F &&f)
+static int with_art_rows(int nx, int ny, F &&f)
 {
+    const int side = std::max(nx, ny);
     if (side <= kArtRayThreads) return f(k_art<1>);
-    if (side <= 2 * kArtRayThreads) return f(k_art<2>);
+    if (side <= 2 * kArtRayThreads || std::min(nx, ny) <= 512 || nx + ny <= 1536) return f(k_art<2>);
     return f(k_art<4>);
 }
 
-int art_max_blocks(int side, int *out)
+int art_max_blocks(int nx, int ny, int *out)
 {
-    return with_art_rows(side, [&](auto *kernel) { return resident_blocks((const void *)kernel, kArtRayThreads, 0, out); });
+    return with_art_rows(nx, ny, [&](auto *kernel) { return resident_blocks((const void *)kernel, kArtRayThreads, 0, out); });
 }
 
 int launch_art_init(const Prob *d_prob, double r, long long rays, cudaStream_t st)
@@ -281,7 +287,7 @@ int launch_art_init(const Prob *d_prob, double r, long long rays, cudaStream_t s
     return SUPCG_OK;
 }
 
-int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st)
+int launch_art(const Prob *d_prob, int nx, int ny, int cycles, double r, double lam, int S, int blocks, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
@@ -293,7 +299,7 @@ int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, i
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return with_art_rows(side, [&](auto *kernel) -> int {
+    return with_art_rows(nx, ny, [&](auto *kernel) -> int {
         SUPCG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, d_prob, cycles, r, lam, S));
         return SUPCG_OK;
     });

@@ -796,9 +796,9 @@ struct Launch {
 int launch_forward(const Launch &L, const Launch &La, int which, int mode, const Io &io = Io());   // La: every view's items
 int launch_backward(const Launch &L, int mode, int bwin, const Io &io = Io());   // BWD_PLAIN: caller sinogram -> caller image
 int launch_backward2(const Launch &L, int bwin);   // g from r and h from q in one pass
-int art_max_blocks(int side, int *out);   // co-resident blocks of k_art, side the longer one of the image
+int art_max_blocks(int nx, int ny, int *out);   // co-resident blocks of k_art for an image
 int launch_art_init(const Prob *d_prob, double r, long long rays, cudaStream_t st);
-int launch_art(const Prob *d_prob, int side, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
+int launch_art(const Prob *d_prob, int nx, int ny, int cycles, double r, double lam, int S, int blocks, cudaStream_t st);
 int backward_blocks(int nx, int ny, int parts, int ti);
 int backward_pairs_blocks(int nx, int ny, int parts, int ti);
 int launch_backward_pairs(const Launch &L, bool dual, int mode, int bwp, const Io &io);
