@@ -9,7 +9,7 @@
 //
 // Two sinograms over 512^2 / 720 views: 219 -> 161 us and 170 M -> 99 M warp instructions against the general
 // kernel (backprojector.cu), which evaluates every weight twice; one sinogram 166 -> 119 us, eight images of
-// 243^2 / 320 views 168 -> 126.  What is left is latency: 49 % of the issue slots are used, the l1tex data
+// 243^2 / 360 views 168 -> 126.  What is left is latency: 49 % of the issue slots are used, the l1tex data
 // path is 60 % busy, no pipe is above 33 %, and two blocks per SM (128 registers) are all that fit.
 #include "backward.cuh"
 
@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward_pairs(co
 #pragma unroll
     for (int h = 0; h < NS * PX / 2; ++h) part2[h] = comp2[h] = pk2(0.0f, 0.0f);
 
+    const float *sino = P.r;
     const void *user = io.in + (size_t)pi * io.in_step;
     const int Up = P.Up;
     // tile corners in pixel-centre coordinates, of the left side
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward_pairs(co
                         for (int k = 0; k < 2; ++k)
                             if (ub + k < P.U) y[a][k] = load_user(user, o + k, io.storage);
                     } else {
-                        const float *sn = (DUAL && (a & 1)) ? P.q : P.r;
+                        const float *sn = (DUAL && (a & 1)) ? P.q : sino;
                         const float2 f = __ldg(reinterpret_cast<const float2 *>(sn + (size_t)v * Up + ub));
                         y[a][0] = f.x; y[a][1] = f.y;
                     }
