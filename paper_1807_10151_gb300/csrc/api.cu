@@ -680,7 +680,7 @@ static int ws_create(const std::vector<supcg_geometry> &gs, Workspace **out)
     }
     if (w->smem_rows > 200 * 1024 || w->smem_cols > 200 * 1024) { delete w; return SUPCG_ERR_UNSUPPORTED; }
     // S_TV on resident tiles when all of them fit the device at once, in the lowest tiles that do (32, 64 or 128
-    // rows; two blocks per SM).  Lower tiles have less work per block between two barriers: K = 40 at 384^2
+    // rows; two blocks per SM).  Lower tiles have less work per block between two barriers: a call with K = 40 at 384^2
     // takes 289, 329 and 426 us with them, at 512^2 338, 338 and 426; where only 64 and 128 rows fit, 640^2
     // 412 and 429; where only 128 do, 1024^2 569.  In memory: 723, 853, 974 and 1308 us.
     for (int ti : {32, 64, 128}) {

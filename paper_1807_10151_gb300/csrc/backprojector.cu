@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kBwdThreads, DUAL ? 2 : 3) k_backward(const Pr
     // per pixel: FP32 sum of up to four views (t2), folded into a Kahan-compensated pair (part, comp)
     // that runs over all views, FP64 only for the final value (the FP64 pipe is narrow).  The views are
     // issue-bound, so all three are kept as pixel pairs and the fold takes half the instructions; it
-    // also ends the repacking that spilled 28 to 112 bytes (171.9 -> 168.3 us for eight 243^2 / 320)
+    // also ends the repacking that spilled 28 to 112 bytes (171.9 -> 168.3 us for eight 243^2 / 360)
     uint64_t part2[NS * PX / 2], comp2[NS * PX / 2], t2[NS * PX / 2];
 #pragma unroll
     for (int h = 0; h < NS * PX / 2; ++h) t2[h] = part2[h] = comp2[h] = pk2(0.0f, 0.0f);

@@ -734,7 +734,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
     return false;
 }
 
-// 2-D tiled TMA load of box (x0 = innermost coordinate, y0) into shared memory.
+// 3-D and 2-D tiled TMA loads of the box at (x0 = innermost coordinate, y0, z0) into shared memory.
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *tm, int x0, int y0, int z0, uint64_t *bar)
 {
     asm volatile(

@@ -588,8 +588,9 @@ __global__ void __launch_bounds__(kTvThreads, 3) k_stv(const Prob *__restrict__ 
 // pixels below and to the right of it in shared memory.  A pixel's values (y~, its
 // term, tbar) are those of k_stv bit for bit: which kernel a problem takes depends on
 // the other problems of its launch.  The two add up the same terms in another order.
-// Measured, K = 40 at 512^2 (one call): 867 -> 364 us, 6.6 us per step; a grid barrier is
-// about 1.4 us of it, the FP64 sum over the blocks' partials 1 us.
+// Measured, K = 40 at 512^2 (one call): 853 -> 338 us, 8.4 us per step; a grid barrier is
+// about 1.4 us of it, the FP64 sum over the blocks' partials 1 us, and the rest some eight block
+// barriers with the short passes between them.
 constexpr int kStvThreads = 512, kStvWarps = kStvThreads / 32;
 
 template <int TI>
@@ -618,7 +619,7 @@ __device__ __forceinline__ void stv_ring(int k, int &i, int &j)
 
 // The step scalars of one thread.  An FP64 instruction holds the SM's FP64 pipe for about 38 cycles per warp
 // that issues it; inlined, these were turned into predicated code that every warp issued (350 FP64
-// instructions per step and block, the pipe 85 % busy: 456 us for 40 steps at 512^2 against 364).
+// instructions per step and block, the pipe 85 % busy: a quarter longer for 40 steps at 512^2).
 struct StvScalars {
     double apow, gap;   // a^l (Scal::apow), gamma a^l
     float gh, gl;       // gamma a^l as two FP32 parts
