@@ -387,8 +387,8 @@ long long supcg_kernel_launches(void);
  * bound in the paper; here it runs on the device in one cooperative launch
  * whose blocks meet at grid barriers, and ART's ray classes (Sec. 3.4) meet
  * at the same kind of barrier.  Each wait polls a flag at most `polls` times
- * (each poll sleeps about 64 ns; the default, 2^24 polls, is a second or
- * two) and then gives up: the kernel records SUPCG_ERR_TIMEOUT, leaves, and
+ * (a poll takes about a quarter of a microsecond; the default, 2^24 polls, is
+ * three to four seconds) and then gives up: the kernel records SUPCG_ERR_TIMEOUT, leaves, and
  * the call returns that status (the context stays usable and the next call
  * starts from a clean barrier).  The setting is process-wide and read by
  * every call when it starts.  The paper has no counterpart.
